@@ -240,8 +240,7 @@ __global__ void __launch_bounds__(kAdjThreads, sizeof(C) == 4 ? LBM_ADJ_MINB_F32
     // boundary transpose and link gradients (Eq. 2.13)
     if (cls == kBoundary) {
       C gp[Q];
-      C drho;
-      collide<L, C>(g, gp, sa, drho);
+      collide<L, C>(g, gp, sa);
       const LinkCoef<C> *coef = static_cast<const LinkCoef<C> *>(sa.geo.coef);
       const int bi = a.bidx[n];
       const uint32_t mask = a.bmask[bi];
@@ -349,9 +348,7 @@ __global__ void __launch_bounds__(kAdjThreads, sizeof(C) == 4 ? 6 : 3)
   }
 #pragma unroll
   for (int i = 0; i < Q; ++i) g[i] = fin[(long long)i * N + n];
-  C drho;
-  collide<L, C>(g, gp, sa, drho);
-  if (!(fabs(drho) < C(1e6))) atomicOr(sa.status, 1);
+  if (collide<L, C>(g, gp, sa)) atomicOr(sa.status, 1);
   const bool inside = x > 0 && x < a.nx - 1 && y > 0 && y < a.ny - 1 &&
                       (L::D == 2 || (z > 0 && z < a.nz - 1));
   if (inside) {

@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "../../include/lbm.h"
+#include "fixed.cuh"
 #include "lattice.h"
 #include "lbm_internal.h"
 
@@ -214,6 +215,7 @@ static void refresh_args(lbm_ctx *c) {
         if (!L::conserved(k)) a.sn[k] = C(c->s[k] / row_norm2<L>(k));
       for (int k = 0; k < 3; ++k) a.F[k] = C(c->rho0 * c->g[k] / L::kNormJ);
       if (L::D == 2) a.F[2] = C(0);
+      if constexpr (sizeof(C) == 8) a.fx = fx_args<L>(c->s, c->rho0, a.F);
       return 0;
     });
     a.inv_rho0 = C(1.0 / c->rho0);

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <type_traits>
 
 namespace lbm {
 
@@ -91,6 +92,21 @@ inline long long slot_stride(long long N) { return (N + 63) / 64 * 64; }
 // (each poll suspends for at most 1 ms: about 1 s in all)
 constexpr int kWaitLimitDefault = 1000;
 
+// Constants of the fixed-point collision of FP64 storage (fixed.cuh), from the host
+// (fill_fixed_args in lbm_capi.cu): a factor in [0, 1/4] as a multiple of 2^-64 in two
+// halves, the low one signed.
+struct FixedCoef {
+  int hi, lo;
+};
+struct FixedArgs {
+  FixedCoef row[19];         // fx_row_scale s_k / |M_k|^2 of the relaxed rows
+  FixedCoef inv_rho0;        // mantissa of 1/rho0 in (1/2, 1] over 4
+  int quad_shift;            // right shift of j_a j_b products, plus the block exponent
+  int max_exp;               // largest biased exponent of a block (below 0: none)
+  int force_hi;              // high word of the largest force component
+};
+struct NoFixedArgs {};
+
 template <class C>
 struct SweepArgs {
   void *pop;                 // population i of node n at pop[i*S + n]
@@ -116,6 +132,7 @@ struct SweepArgs {
   // when non-null, the sweep also writes every fluid node's pre-collision
   // deviations g_i(x, t) here, natural layout save[i*N + n] (adjoint recomputation)
   C *save = nullptr;
+  std::conditional_t<sizeof(C) == 8, FixedArgs, NoFixedArgs> fx;
 };
 
 // launchers (return cudaGetLastError() of the launch)

@@ -31,8 +31,7 @@ __global__ void two_node_pre_kernel(const SweepArgs<typename Storage<T>::C> sa, 
   C g[Q], gp[Q];
 #pragma unroll
   for (int q = 0; q < Q; ++q) g[q] = C(Storage<T>::load(population_address<L, T>(q, e.xl, odd, a)));
-  C drho;
-  collide<L, C>(g, gp, sa, drho);
+  collide<L, C>(g, gp, sa);
   // gp[d] for the runtime direction d, without a local-memory table
   C fl_next = C(0);
 #pragma unroll
