@@ -7,6 +7,7 @@
 // of x - e_i, or in the link buffer for a cut link.  They compute in double
 // whatever the storage type.
 #include "common.cuh"
+#include "node_sums.cuh"
 
 namespace lbm {
 
@@ -69,38 +70,41 @@ __global__ void set_pop_kernel(AuxArgs a, const double *f) {
   }
 }
 
-// density deviation and momentum of node n
+// Density and velocity of every node.  One thread per node; the velocities of a warp (D
+// doubles per node, node-major) pass through shared memory, so that each store covers
+// whole sectors.
+constexpr int kMomThreads = 256;
 template <class L, class T>
-__device__ __forceinline__ void node_moments(const AuxArgs &a, const T *pop, long long n, bool odd,
-                                             double &drho, double (&j)[3]) {
-  drho = 0;
-  j[0] = j[1] = j[2] = 0;
+__global__ void __launch_bounds__(kMomThreads) moments_kernel(AuxArgs a, bool odd, double *rho, double *u) {
+  constexpr int D = L::D;
+  __shared__ double sh[kMomThreads / 32][32 * D];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (long long base = (blockIdx.x * (long long)kMomThreads) + warp * 32; base < a.N;
+       base += (long long)gridDim.x * kMomThreads) {
+    const int n = (int)base + lane;
+    double r = quiet_nan(), v[3] = {r, r, r};
+    const int cls = base + lane < a.N ? (int)a.cls[n] : (int)kSolid;
+    if (cls != kSolid) {
+      typename Storage<T>::C g[L::Q];
+      load_node<L, T>(g, n, cls, odd, a);
+      double drho, j[3];
+      node_sums<L>(g, drho, j);
+      r = a.rho0 + drho;
 #pragma unroll
-  for (int i = 0; i < L::Q; ++i) {
-    const double g = (double)Storage<T>::load(population_address<L, T>(i, n, odd, a));
-    drho += g;
-    j[0] += L::ex(i) * g;
-    j[1] += L::ey(i) * g;
-    j[2] += L::ez(i) * g;
-  }
-}
-
-template <class L, class T>
-__global__ void moments_kernel(AuxArgs a, bool odd, double *rho, double *u) {
-  const T *pop = static_cast<const T *>(a.pop);
-  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < a.N;
-       n += (long long)gridDim.x * blockDim.x) {
-    if (a.cls[n] == kSolid) {
-      if (rho) rho[n] = quiet_nan();
-      if (u)
-        for (int k = 0; k < L::D; ++k) u[n * L::D + k] = quiet_nan();
-      continue;
+      for (int k = 0; k < D; ++k) v[k] = velocity(j[k], a, k);
     }
-    double drho, j[3];
-    node_moments<L, T>(a, pop, n, odd, drho, j);
-    if (rho) rho[n] = a.rho0 + drho;
-    if (u)
-      for (int k = 0; k < L::D; ++k) u[n * L::D + k] = j[k] / a.rho0 + 0.5 * a.g[k];
+    if (rho && base + lane < a.N) rho[n] = r;
+    if (u) {
+#pragma unroll
+      for (int k = 0; k < D; ++k) sh[warp][lane * D + k] = v[k];
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        const long long o = base * D + k * 32 + lane;
+        if (o < a.N * D) u[o] = sh[warp][k * 32 + lane];
+      }
+      __syncwarp();
+    }
   }
 }
 
@@ -110,15 +114,17 @@ template <class L, class T>
 __global__ void __launch_bounds__(kNormThreads)
     norm_partials_kernel(AuxArgs a, bool odd, const double *u_ref, double *u_prev,
                          double *partials) {
-  const T *pop = static_cast<const T *>(a.pop);
   double acc[kNormFields];
 #pragma unroll
   for (int k = 0; k < kNormFields; ++k) acc[k] = 0.0;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < a.N;
        n += (long long)gridDim.x * blockDim.x) {
-    if (a.cls[n] == kSolid) continue;
+    const int cls = a.cls[n];
+    if (cls == kSolid) continue;
+    typename Storage<T>::C g[L::Q];
+    load_node<L, T>(g, (int)n, cls, odd, a);
     double drho, j[3];
-    node_moments<L, T>(a, pop, n, odd, drho, j);
+    node_sums<L>(g, drho, j);
     const double rho = a.rho0 + drho;
     if (!isfinite(rho)) acc[9] += 1.0;
     acc[3] += rho;
@@ -127,7 +133,7 @@ __global__ void __launch_bounds__(kNormThreads)
     acc[6] += j[2];
 #pragma unroll
     for (int k = 0; k < L::D; ++k) {
-      const double uk = j[k] / a.rho0 + 0.5 * a.g[k];
+      const double uk = velocity(j[k], a, k);
       if (u_ref) {
         const double r = u_ref[n * L::D + k];
         const double df = r - uk;
@@ -162,16 +168,20 @@ __global__ void __launch_bounds__(kNormThreads)
   }
 }
 
-__global__ void norm_finish_kernel(const double *partials, int n_blocks, double *out) {
-  // one block; thread k < kNormFields reduces field k over the blocks in order
-  const int k = threadIdx.x;
-  if (k >= kNormFields) return;
-  double v = (k == 2) ? 0.0 : 0.0;
-  for (int b = 0; b < n_blocks; ++b) {
+// warp k reduces field k over the blocks' records, in a fixed order
+__global__ void __launch_bounds__(32 * kNormFields) norm_finish_kernel(const double *partials, int n_blocks,
+                                                                     double *out) {
+  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double v = 0.0;
+  for (int b = lane; b < n_blocks; b += 32) {
     const double w = partials[(long long)b * kNormFields + k];
     v = (k == 2) ? fmax(v, w) : v + w;
   }
-  out[k] = v;
+  for (int o = 16; o > 0; o >>= 1) {
+    const double w = __shfl_down_sync(0xffffffffu, v, o);
+    v = (k == 2) ? fmax(v, w) : v + w;
+  }
+  if (lane == 0) out[k] = v;
 }
 
 int aux_blocks(long long N) {
@@ -232,7 +242,7 @@ cudaError_t launch_moments(int lattice, int precision, const AuxArgs &a, bool od
     using L = decltype(lat);
     return with_storage(precision, [&](auto *tp) {
       using T = std::remove_pointer_t<decltype(tp)>;
-      moments_kernel<L, T><<<aux_blocks(a.N), 256, 0, st>>>(a, odd, rho, u);
+      moments_kernel<L, T><<<aux_blocks(a.N), kMomThreads, 0, st>>>(a, odd, rho, u);
       return cudaGetLastError();
     });
   });
@@ -254,7 +264,7 @@ cudaError_t launch_norm_partials(int lattice, int precision, const AuxArgs &a, b
 
 cudaError_t launch_norm_finish(const double *partials, int n_blocks, double *out,
                                cudaStream_t st) {
-  norm_finish_kernel<<<1, 32, 0, st>>>(partials, n_blocks, out);
+  norm_finish_kernel<<<1, 32 * kNormFields, 0, st>>>(partials, n_blocks, out);
   return cudaGetLastError();
 }
 

@@ -181,6 +181,8 @@ static AuxArgs aux_args(const lbm_ctx *c) {
   a.boff = c->boff;
   a.lnk = c->lnk;
   a.rho0 = c->rho0;
+  int e = 0;
+  a.inv_rho0 = std::frexp(c->rho0, &e) == 0.5 ? 1.0 / c->rho0 : 0.0;
   for (int k = 0; k < 3; ++k) a.g[k] = c->g[k];
   return a;
 }

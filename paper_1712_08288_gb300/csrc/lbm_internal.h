@@ -153,6 +153,7 @@ struct AuxArgs {
   const int32_t *boff;
   const void *lnk;
   double rho0;
+  double inv_rho0;           // 1 / rho0 where rho0 is a power of two, else 0
   double g[3];
 };
 

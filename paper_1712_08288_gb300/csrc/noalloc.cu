@@ -20,14 +20,14 @@
 
 #include "../../include/lbm.h"
 #include "common.cuh"
+#include "node_sums.cuh"
 
 namespace lbm {
 namespace {
 
 constexpr int kNoAllocThreads = 256;
 constexpr int kNoAllocBlocks = 1024;                     // partial records in the array
-constexpr long long kNoAllocNodesPerBlock = 32768;       // nodes reduced by one block
-constexpr long long kNoAllocMaxNodes = kNoAllocBlocks * kNoAllocNodesPerBlock;  // 33,554,432
+constexpr long long kNoAllocMaxNodes = 33554432;         // documented limit of the entry point
 constexpr int kFields = 8;  // sum|u_ref-u|^2, sum|u_ref|^2, max|u_ref-u|, sum rho, sum j (3), non-finite
 
 static __device__ __align__(256) double g_noalloc_partials[kNoAllocBlocks * kFields];
@@ -38,20 +38,14 @@ __global__ void __launch_bounds__(kNoAllocThreads)
   double acc[kFields];
 #pragma unroll
   for (int k = 0; k < kFields; ++k) acc[k] = 0.0;
-  const long long begin = (long long)blockIdx.x * kNoAllocNodesPerBlock;
-  long long end = begin + kNoAllocNodesPerBlock;
-  if (end > a.N) end = a.N;
-  for (long long n = begin + threadIdx.x; n < end; n += kNoAllocThreads) {
-    if (a.cls[n] == kSolid) continue;
-    double drho = 0.0, j[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-    for (int i = 0; i < L::Q; ++i) {
-      const double g = (double)Storage<T>::load(population_address<L, T>(i, n, odd, a));
-      drho += g;
-      j[0] += L::ex(i) * g;
-      j[1] += L::ey(i) * g;
-      j[2] += L::ez(i) * g;
-    }
+  for (long long n = blockIdx.x * (long long)kNoAllocThreads + threadIdx.x; n < a.N;
+       n += (long long)gridDim.x * kNoAllocThreads) {
+    const int cls = a.cls[n];
+    if (cls == kSolid) continue;
+    typename Storage<T>::C g[L::Q];
+    load_node<L, T>(g, (int)n, cls, odd, a);
+    double drho, j[3];
+    node_sums<L>(g, drho, j);
     const double rho = a.rho0 + drho;
     if (!isfinite(rho)) acc[7] += 1.0;
     acc[3] += rho;
@@ -61,7 +55,7 @@ __global__ void __launch_bounds__(kNoAllocThreads)
     if (u_ref) {
 #pragma unroll
       for (int k = 0; k < L::D; ++k) {
-        const double uk = j[k] / a.rho0 + 0.5 * a.g[k];
+        const double uk = velocity(j[k], a, k);
         const double df = u_ref[n * L::D + k] - uk;
         acc[0] += df * df;
         acc[1] += u_ref[n * L::D + k] * u_ref[n * L::D + k];
@@ -89,21 +83,23 @@ __global__ void __launch_bounds__(kNoAllocThreads)
   }
 }
 
-// out: l2_rel, linf, mass, mom_x, mom_y, mom_z, non-finite count
-__global__ void noalloc_finish_kernel(const double *partials, int n_blocks, bool have_ref,
-                                      double *out) {
+// out: l2_rel, linf, mass, mom_x, mom_y, mom_z, non-finite count; warp k reduces field k
+__global__ void __launch_bounds__(32 * kFields) noalloc_finish_kernel(const double *partials, int n_blocks,
+                                                                    bool have_ref, double *out) {
   __shared__ double tot[kFields];
-  const int k = threadIdx.x;
-  if (k < kFields) {
-    double v = 0.0;
-    for (int b = 0; b < n_blocks; ++b) {
-      const double w = partials[b * kFields + k];
-      v = (k == 2) ? fmax(v, w) : v + w;
-    }
-    tot[k] = v;
+  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double v = 0.0;
+  for (int b = lane; b < n_blocks; b += 32) {
+    const double w = partials[b * kFields + k];
+    v = (k == 2) ? fmax(v, w) : v + w;
   }
+  for (int o = 16; o > 0; o >>= 1) {
+    const double w = __shfl_down_sync(0xffffffffu, v, o);
+    v = (k == 2) ? fmax(v, w) : v + w;
+  }
+  if (lane == 0) tot[k] = v;
   __syncthreads();
-  if (k == 0) {
+  if (threadIdx.x == 0) {
     const double nan = __longlong_as_double(0x7ff8000000000000LL);
     out[0] = have_ref ? sqrt(tot[0]) / sqrt(tot[1]) : nan;
     out[1] = have_ref ? tot[2] : nan;
@@ -156,7 +152,9 @@ int error_norms_noalloc(int device, int lattice, int precision, const AuxArgs &a
     *why = cudaGetErrorString(e);
     return LBM_ECUDA;
   }
-  const int n_blocks = (int)((a.N + kNoAllocNodesPerBlock - 1) / kNoAllocNodesPerBlock);
+  // one record per block; as many blocks as the array has records, fewer on small grids
+  const long long want = (a.N + kNoAllocThreads - 1) / kNoAllocThreads;
+  const int n_blocks = (int)(want < kNoAllocBlocks ? want : kNoAllocBlocks);
   e = with_lattice(lattice, [&](auto lat) {
     using L = decltype(lat);
     return with_storage(precision, [&](auto *tp) {
@@ -166,7 +164,7 @@ int error_norms_noalloc(int device, int lattice, int precision, const AuxArgs &a
     });
   });
   if (e == cudaSuccess) {
-    noalloc_finish_kernel<<<1, 32, 0, st>>>(scratch, n_blocks, u_ref != nullptr, out);
+    noalloc_finish_kernel<<<1, 32 * kFields, 0, st>>>(scratch, n_blocks, u_ref != nullptr, out);
     e = cudaGetLastError();
   }
   if (e != cudaSuccess) {

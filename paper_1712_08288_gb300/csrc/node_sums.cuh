@@ -1,0 +1,140 @@
+// node_sums.cuh -- a node's populations at either time parity and their FP64 sums rho
+// and j, for the read-out kernels (moments, error norms).
+//
+// The sums run in 64-bit integers aligned to the node's largest population: in FP64 they
+// cost some 60 instructions (conversions and additions) at one warp instruction in 64 cycles per
+// quarter SM, several times the time that the populations take to arrive from memory.
+// 32-bit and 16-bit storage: every population within 2^33 of the largest is exact, so the
+// sums are too; smaller ones lose less than 2^-57 of the largest.  FP64 storage: one unit
+// is 1/32 of an ulp of the largest population, where an FP64 sum rounds each
+// addition.  Nodes with a non-finite value, or with none above the small end of
+// the range, take FP64 sums.
+#pragma once
+
+#include "common.cuh"
+#include "fixed.cuh"
+
+namespace lbm {
+
+// How a read-out kernel walks the grid: node coordinates by 32-bit arithmetic.
+template <int D>
+struct NodeAt {
+  int x, y, z;
+  bool inside;   // no neighbour across a periodic face
+  __device__ __forceinline__ NodeAt(int n, const AuxArgs &a) {
+    const unsigned r = (unsigned)n / (unsigned)a.nx;
+    x = n - (int)r * a.nx;
+    z = (int)(r / (unsigned)a.ny);
+    y = (int)r - z * a.ny;
+    inside = x > 0 && x < a.nx - 1 && y > 0 && y < a.ny - 1 && (D == 2 || (z > 0 && z < a.nz - 1));
+  }
+};
+
+// f_i(x_n, t) - w_i rho0 for all i, in the compute type (population_address() for one)
+template <class L, class T>
+__device__ __forceinline__ void load_node(typename Storage<T>::C (&g)[L::Q], int n, int cls, bool odd,
+                                          const AuxArgs &a) {
+  const T *pop = static_cast<const T *>(a.pop) + n;
+  if (!odd) {
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) g[i] = Storage<T>::load(pop + (long long)i * a.S);
+    return;
+  }
+  const NodeAt<L::D> at(n, a);
+  if (at.inside) {
+    const long long sx = a.nx, sxy = (long long)a.nx * a.ny;
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i)
+      g[i] = Storage<T>::load(pop + ((long long)L::opp(i) * a.S - L::ex(i) - L::ey(i) * sx - L::ez(i) * sxy));
+  } else {
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i)
+      g[i] = Storage<T>::load(pop - n + (long long)L::opp(i) * a.S +
+                              wrap_index(at.x, at.y, at.z, -L::ex(i), -L::ey(i), -L::ez(i), a.nx, a.ny, a.nz, a.sy, a.sz));
+  }
+  if (cls == kBoundary) {
+    const int b = a.bidx[n];
+    const uint32_t m = a.bmask[b];
+    const T *lnk = static_cast<const T *>(a.lnk) + a.boff[b];
+#pragma unroll
+    for (int d = 1; d < L::Q; ++d)
+      if ((m >> d) & 1u) g[L::opp(d)] = Storage<T>::load(lnk + __popc(m & ((1u << d) - 1u)));
+  }
+}
+
+// sums of the integers, times 2^scale
+template <class L>
+__device__ __forceinline__ void scaled_sums(const i64 (&v)[L::Q], int scale, double &drho, double (&j)[3]) {
+  i64 m[L::Q];
+  fmoments<i64>(L{}, v, m);   // rho and j are used, the rest is never computed
+  auto to = [&](i64 x) {
+    const double d = (double)x;
+    return __hiloint2double(x != 0 ? __double2hiint(d) + (scale << 20) : 0, __double2loint(d));
+  };
+  drho = to(m[0]);
+  j[0] = to(m[3]);
+  j[1] = to(m[5]);
+  j[2] = L::D == 3 ? to(m[7]) : 0.0;
+}
+
+template <class L, class C>
+__device__ __forceinline__ void plain_sums(const C (&g)[L::Q], double &drho, double (&j)[3]) {
+  drho = j[0] = j[1] = j[2] = 0.0;
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) {
+    const double v = (double)g[i];
+    drho += v;
+    if (L::ex(i) != 0) j[0] += L::ex(i) * v;
+    if (L::ey(i) != 0) j[1] += L::ey(i) * v;
+    if (L::ez(i) != 0) j[2] += L::ez(i) * v;
+  }
+}
+
+template <class L>
+__device__ __forceinline__ void node_sums(const float (&g)[L::Q], double &drho, double (&j)[3]) {
+  constexpr int kTop = 57;        // 19 (2^58) < 2^63
+  unsigned mx = 0;
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) mx = max(mx, __float_as_uint(g[i]) & 0x7fffffffu);
+  const int E = (int)(mx >> 23);
+  if (mx != 0 && (E < 64 || E == 255)) {   // below 64 a subnormal number could count
+    plain_sums<L>(g, drho, j);
+    return;
+  }
+  i64 v[L::Q];
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) {
+    const unsigned b = __float_as_uint(g[i]);
+    const int d = max(E, 64) - (int)((b >> 23) & 0xffu);
+    const u64 top = (u64)(((b & 0x7fffffu) | 0x800000u) << (kTop - 23 - 32)) << 32;
+    const i64 s = (i64)((int)b >> 31);
+    v[i] = ((i64)fx_shr(top, d) ^ s) - s;
+  }
+  scaled_sums<L>(v, max(E, 64) - 127 - kTop, drho, j);
+}
+
+template <class L>
+__device__ __forceinline__ void node_sums(const double (&g)[L::Q], double &drho, double (&j)[3]) {
+  constexpr int kTop = 57;
+  int mx = 0;
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) mx = max(mx, __double2hiint(g[i]) & 0x7fffffff);
+  const int E = mx >> 20;
+  if (mx != 0 && (E < kFxMinExp || E == 2047)) {
+    plain_sums<L>(g, drho, j);
+    return;
+  }
+  i64 v[L::Q];
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) v[i] = fx_from<kTop>(g[i], max(E, kFxMinExp));
+  scaled_sums<L>(v, max(E, kFxMinExp) - 1023 - kTop, drho, j);
+}
+
+// velocity component: j / rho0 + g / 2.  A power of two is divided by exactly by its
+// reciprocal (one instruction instead of a division's dozen).
+__device__ __forceinline__ double velocity(double j, const AuxArgs &a, int k) {
+  const double u = a.inv_rho0 != 0.0 ? j * a.inv_rho0 : j / a.rho0;
+  return a.g[k] != 0.0 ? u + 0.5 * a.g[k] : u;
+}
+
+}  // namespace lbm
