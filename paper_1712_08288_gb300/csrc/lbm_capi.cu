@@ -86,6 +86,7 @@ struct lbm_ctx {
   uint32_t *bmask = nullptr;
   int32_t *boff = nullptr;
   uint32_t *rec32 = nullptr;    // packed records of boundary nodes
+  uint16_t *ldesc = nullptr;    // link descriptors of the link-parallel boundary
   void *coef = nullptr;
   void *lnk = nullptr;          // boundary values carried from an even to an odd step
   int *status = nullptr;
@@ -201,6 +202,7 @@ static void refresh_args(lbm_ctx *c) {
   DevGeometry geo;
   geo.cls = c->cls; geo.bidx = c->bidx; geo.bmask = c->bmask; geo.boff = c->boff;
   geo.rec32 = c->rec32;
+  geo.ldesc = c->ldesc;
   geo.coef = c->coef;
   geo.lnk = c->lnk;
   auto fill = [&](auto &a) {
@@ -357,18 +359,53 @@ static void free_geometry(lbm_ctx *c) {
   cudaFree(c->lnk); c->lnk = nullptr;
 }
 
+// A tile list in the device form (TileDesc of every tile, then TileLinks), and back.
+static cudaError_t put_tiles(const std::vector<HostTile> &t, TileDesc **dev) {
+  const size_t n = t.size(), bytes = (sizeof(TileDesc) + sizeof(TileLinks)) * n;
+  cudaError_t e = cudaMalloc((void **)dev, std::max<size_t>(sizeof(TileDesc), bytes));
+  if (e != cudaSuccess) *dev = nullptr;
+  if (e != cudaSuccess || n == 0) return e;
+  std::vector<unsigned char> h(bytes);
+  TileDesc *d = reinterpret_cast<TileDesc *>(h.data());
+  TileLinks *k = reinterpret_cast<TileLinks *>(d + n);
+  for (size_t i = 0; i < n; ++i) {
+    d[i] = t[i];
+    k[i] = t[i];
+  }
+  return cudaMemcpy(*dev, h.data(), bytes, cudaMemcpyHostToDevice);
+}
+static cudaError_t get_tiles(const TileDesc *dev, size_t n, std::vector<HostTile> &t) {
+  t.resize(n);
+  if (n == 0) return cudaSuccess;
+  std::vector<unsigned char> h((sizeof(TileDesc) + sizeof(TileLinks)) * n);
+  const cudaError_t e = cudaMemcpy(h.data(), dev, h.size(), cudaMemcpyDeviceToHost);
+  const TileDesc *d = reinterpret_cast<const TileDesc *>(h.data());
+  const TileLinks *k = reinterpret_cast<const TileLinks *>(d + n);
+  for (size_t i = 0; i < n; ++i) {
+    static_cast<TileDesc &>(t[i]) = d[i];
+    static_cast<TileLinks &>(t[i]) = k[i];
+  }
+  return e;
+}
+
 // 64-node tiles cut into 32-node halves; halves without a fluid node are dropped.
 // A half keeps the tile's link-buffer base (its records' offsets are relative to it);
 // the second half's records start after the first half's.  Lanes past a half are
 // marked solid.
-static void half_tiles(const std::vector<TileDesc> &in, std::vector<TileDesc> &out) {
+static void half_tiles(const std::vector<HostTile> &in, std::vector<HostTile> &out) {
   constexpr uint64_t kLo = 0xffffffffull;
   out.clear();
   out.reserve(2 * in.size());
-  for (const TileDesc &d : in) {
-    TileDesc a = d, h = d;
+  for (const HostTile &d : in) {
+    HostTile a = d, h = d;
     a.solid = d.solid | ~kLo;
     a.bnd = d.bnd & kLo;
+    a.k1 = 0;
+    h.l0 = d.l0 + d.k0;
+    h.k0 = d.k1;
+    h.k1 = 0;
+    a.dense = a.k0 > kSparseLinks;
+    h.dense = h.k0 > kSparseLinks;
     h.x0 = d.x0 + 32;
     h.rb = d.rb + __builtin_popcountll(d.bnd & kLo);
     h.solid = (d.solid >> 32) | ~kLo;
@@ -386,17 +423,19 @@ static int upload_tiles(lbm_ctx *c, const uint8_t *solid, const std::vector<uint
   if (c->ny > 65535 || c->nz > 65535)
     return fail(c, LBM_EINVAL, "grid: ny and nz must be below 65536");
   const int nxb = (c->nx + kTileW - 1) / kTileW;
-  std::vector<TileDesc> t;
+  std::vector<HostTile> t;
   t.reserve((size_t)nxb * c->ny * c->nz);
   std::vector<uint32_t> rec32;
+  std::vector<uint16_t> ldesc;
   if (bmask) rec32.reserve(bmask->size());
+  ldesc.reserve((size_t)c->n_links);
   int rb = 0;
   for (int z = 0; z < c->nz; ++z)
     for (int y = 0; y < c->ny; ++y)
       for (int xb = 0; xb < nxb; ++xb) {
         const int x0 = xb * kTileW;
         const long long row = (long long)c->nx * (y + (long long)c->ny * z);
-        TileDesc d{};
+        HostTile d{};
         d.x0 = x0;
         d.yz = y | (z << 16);
         d.rb = rb;
@@ -409,33 +448,38 @@ static int upload_tiles(lbm_ctx *c, const uint8_t *solid, const std::vector<uint
           any = true;
           if (cls && (*cls)[row + x] == kBoundary) {
             const uint32_t m = (*bmask)[rb], off = (uint32_t)(*boff)[rb];
-            if (!d.bnd) d.lb = (int)off;
+            if (!d.bnd) d.lb = d.l0 = (int)off;
+            (k < 32 ? d.k0 : d.k1) += (unsigned short)__builtin_popcount(m);
+            for (int dir = 1; dir < c->Q; ++dir)
+              if ((m >> dir) & 1u) ldesc.push_back((uint16_t)((k & 31) | (dir << kLinkDirShift)));
             d.bnd |= 1ull << k;
             rec32.push_back(m | ((off - (uint32_t)d.lb) << kRecShift));
             ++rb;
           }
         }
+        d.dense = d.k0 > kSparseLinks || d.k1 > kSparseLinks;
         if (any) t.push_back(d);
       }
   c->n_tiles = (int)t.size();
   cudaFree(c->tiles);
   c->tiles = nullptr;
-  std::vector<TileDesc> th;
+  std::vector<HostTile> th;
   half_tiles(t, th);
   c->n_tiles_half = (int)th.size();
   cudaFree(c->tiles_half);
   c->tiles_half = nullptr;
-  CUDA_OR_FAIL(c, cudaMalloc((void **)&c->tiles_half, sizeof(TileDesc) * std::max<size_t>(1, th.size())));
-  if (!th.empty())
-    CUDA_OR_FAIL(c, cudaMemcpy(c->tiles_half, th.data(), sizeof(TileDesc) * th.size(),
-                               cudaMemcpyHostToDevice));
+  CUDA_OR_FAIL(c, put_tiles(th, &c->tiles_half));
   cudaFree(c->rec32);
   c->rec32 = nullptr;
-  CUDA_OR_FAIL(c, cudaMalloc((void **)&c->tiles, sizeof(TileDesc) * std::max<size_t>(1, t.size())));
-  if (!t.empty())
-    CUDA_OR_FAIL(c, cudaMemcpy(c->tiles, t.data(), sizeof(TileDesc) * t.size(), cudaMemcpyHostToDevice));
+  CUDA_OR_FAIL(c, put_tiles(t, &c->tiles));
   CUDA_OR_FAIL(c, cudaMalloc((void **)&c->rec32, sizeof(uint32_t) * rec32.size() + kGuardBytes));
   CUDA_OR_FAIL(c, cudaMemset(c->rec32, 0, sizeof(uint32_t) * rec32.size() + kGuardBytes));
+  cudaFree(c->ldesc);
+  c->ldesc = nullptr;
+  CUDA_OR_FAIL(c, cudaMalloc((void **)&c->ldesc, sizeof(uint16_t) * ldesc.size() + kGuardBytes));
+  CUDA_OR_FAIL(c, cudaMemset(c->ldesc, 0, sizeof(uint16_t) * ldesc.size() + kGuardBytes));
+  if (!ldesc.empty())
+    CUDA_OR_FAIL(c, cudaMemcpy(c->ldesc, ldesc.data(), sizeof(uint16_t) * ldesc.size(), cudaMemcpyHostToDevice));
   if (!rec32.empty())
     CUDA_OR_FAIL(c, cudaMemcpy(c->rec32, rec32.data(), sizeof(uint32_t) * rec32.size(),
                                cudaMemcpyHostToDevice));
@@ -515,6 +559,8 @@ int lbm_destroy(lbm_ctx *c) {
   c->tiles_half = nullptr;
   cudaFree(c->rec32);
   c->rec32 = nullptr;
+  cudaFree(c->ldesc);
+  c->ldesc = nullptr;
   cudaFree(c->partials);
   cudaFree(c->norm_out);
   cudaFree(c->u_ref);
@@ -1280,7 +1326,7 @@ struct lbm_batch {
   std::vector<lbm_ctx *> ctx;
   int lattice = 0, precision = 0, device = 0;
   cudaStream_t stream = nullptr;
-  std::vector<std::vector<TileDesc>> host_tiles;   // per context
+  std::vector<std::vector<HostTile>> host_tiles;   // per context
   std::vector<long long> versions;
   void *inst = nullptr;          // SweepArgs per context (compute type of the precision)
   BatchList lists[kBatchClasses];  // tile lists per kernel class (batch_upload)
@@ -1343,9 +1389,9 @@ static int batch_upload(lbm_batch *b) {
     }
   // the members' tiles in the batch's tile width (64-bit slot indices: 64 only)
   const bool halves = b->tile_w == 32 && !b->big;
-  std::vector<std::vector<TileDesc>> halved(halves ? n : 0);
+  std::vector<std::vector<HostTile>> halved(halves ? n : 0);
   for (int k = 0; k < (halves ? n : 0); ++k) half_tiles(b->host_tiles[k], halved[k]);
-  const std::vector<std::vector<TileDesc>> &mt = halves ? halved : b->host_tiles;
+  const std::vector<std::vector<HostTile>> &mt = halves ? halved : b->host_tiles;
   std::vector<int> ctx_order(n);
   for (int k = 0; k < n; ++k) ctx_order[k] = k;
   if (b->order == 2)
@@ -1355,7 +1401,7 @@ static int batch_upload(lbm_batch *b) {
   b->n_tiles = 0;
   for (int cl = 0; cl < kBatchClasses; ++cl) {
     BatchList &bl = b->lists[cl];
-    std::vector<TileDesc> t;
+    std::vector<HostTile> t;
     std::vector<int> ti;
     if (b->order == 1) {
       // round-robin: one tile of every member of the class in turn
@@ -1373,7 +1419,7 @@ static int batch_upload(lbm_batch *b) {
     } else {
       for (int k : ctx_order)
         if (cls_of[k] == cl)
-          for (const TileDesc &d : mt[k]) {
+          for (const HostTile &d : mt[k]) {
             t.push_back(d);
             ti.push_back(k);
           }
@@ -1385,9 +1431,8 @@ static int batch_upload(lbm_batch *b) {
     bl.n = (int)t.size();
     b->n_tiles += bl.n;
     if (t.empty()) continue;
-    BCUDA(b, cudaMalloc((void **)&bl.tiles, sizeof(TileDesc) * t.size()));
+    BCUDA(b, put_tiles(t, &bl.tiles));
     BCUDA(b, cudaMalloc((void **)&bl.tile_inst, sizeof(int) * ti.size()));
-    BCUDA(b, cudaMemcpy(bl.tiles, t.data(), sizeof(TileDesc) * t.size(), cudaMemcpyHostToDevice));
     BCUDA(b, cudaMemcpy(bl.tile_inst, ti.data(), sizeof(int) * ti.size(), cudaMemcpyHostToDevice));
   }
   return LBM_OK;
@@ -1415,10 +1460,7 @@ static int batch_refresh_if_needed(lbm_batch *b) {
   // geometry may have changed: fetch the tile lists again
   for (size_t k = 0; k < b->ctx.size(); ++k) {
     lbm_ctx *c = b->ctx[k];
-    b->host_tiles[k].resize(c->n_tiles);
-    if (c->n_tiles)
-      BCUDA(b, cudaMemcpy(b->host_tiles[k].data(), c->tiles, sizeof(TileDesc) * c->n_tiles,
-                          cudaMemcpyDeviceToHost));
+    BCUDA(b, get_tiles(c->tiles, c->n_tiles, b->host_tiles[k]));
   }
   int rc = batch_upload(b);
   if (rc == LBM_OK) rc = batch_upload_args(b);

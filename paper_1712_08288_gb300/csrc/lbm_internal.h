@@ -6,7 +6,6 @@
 #include <stdint.h>
 
 #include <string>
-#include <type_traits>
 
 namespace lbm {
 
@@ -46,6 +45,19 @@ struct alignas(16) TileDesc {
   int x0, yz, rb, lb;
   unsigned long long solid, bnd;
 };
+// A tile's links for the link-parallel boundary (FP64 storage): first link, counts of
+// the two 32-node halves (a half tile has one), and whether a half has more than
+// kSparseLinks.  A list of n tiles on the device is n TileDesc, then n TileLinks (apart,
+// since the sweeps that do not need them lose 3 % to the longer descriptors).
+struct alignas(16) TileLinks {
+  int l0;
+  unsigned short k0, k1;
+  int dense, pad;
+};
+struct HostTile : TileDesc, TileLinks {};
+constexpr int kSparseLinks = 64;
+// descriptor of a link: node within its 32-node half in bits 0..4, direction above
+constexpr int kLinkDirShift = 5;
 // packed record of a boundary node: cut-direction mask in bits 0..18, offset of
 // its first link relative to the tile's lb in bits 19..31
 constexpr int kRecShift = 19;
@@ -65,6 +77,7 @@ struct DevGeometry {
   const uint32_t *bmask = nullptr;
   const int32_t *boff = nullptr;
   const uint32_t *rec32 = nullptr; // packed records (see TileDesc), in node order
+  const uint16_t *ldesc = nullptr; // link descriptors, in link order (guard bytes after the end)
   const void *coef = nullptr;      // 4 coefficients per link, compute type
   void *lnk = nullptr;             // one storage element per link (see below)
 };
@@ -105,10 +118,15 @@ struct FixedArgs {
   int max_exp;               // largest biased exponent of a block (below 0: none)
   int force_hi;              // high word of the largest force component
 };
-struct NoFixedArgs {};
+template <class C>
+struct FixedPart {};
+template <>
+struct FixedPart<double> {
+  FixedArgs fx;
+};
 
 template <class C>
-struct SweepArgs {
+struct SweepArgs : FixedPart<C> {
   void *pop;                 // population i of node n at pop[i*S + n]
   long long N;               // nodes
   long long S;               // slot stride
@@ -132,7 +150,6 @@ struct SweepArgs {
   // when non-null, the sweep also writes every fluid node's pre-collision
   // deviations g_i(x, t) here, natural layout save[i*N + n] (adjoint recomputation)
   C *save = nullptr;
-  std::conditional_t<sizeof(C) == 8, FixedArgs, NoFixedArgs> fx;
 };
 
 // launchers (return cudaGetLastError() of the launch)

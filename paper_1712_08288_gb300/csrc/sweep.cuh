@@ -497,6 +497,20 @@ static_assert((StageShape<float>::kWidth * sizeof(float)) % 16 == 0, "window str
 static_assert((StageShape<double>::kWidth * sizeof(double)) % 16 == 0, "window stride");
 static_assert((StageShape<__half>::kWidth * sizeof(__half)) % 16 == 0, "window stride");
 
+// Cut links of FP64 storage go link by link over the lanes of the warp, other storage node by
+// node.  In FP64 a boundary value takes 5 instructions of 64 issue cycles each, and a
+// lane per node runs them for every cut direction that any node of the warp has (some 8
+// on a curved wall, a few lanes each); a lane per link runs them once for up to 32
+// links: D3Q19 pipe L = 128, 164 -> 125 us a step; D2Q9 511^2, 14.4 -> 12.0.  The
+// exchange between the lanes of nodes and links costs more than it saves where arithmetic is cheap
+// (FP32: pipe L = 256, 271 -> 288 us; ensemble of 32 annuli, 62 -> 69).
+template <class T>
+__host__ __device__ constexpr bool link_parallel() {
+  return sizeof(T) == 8;
+}
+static_assert(StageShape<double, 32>::kRecs * 4 >= kSparseLinks * 2 + 16 && StageShape<double>::kRecs * 4 >= 2 * kSparseLinks * 2 + 16,
+              "the link descriptors of a sparse tile fit the record window");
+
 // aligned-down source of a window and the element offset of its first element
 template <class E>
 __device__ __forceinline__ const char *align16(const E *p, int &off_elems) {
@@ -516,7 +530,7 @@ __device__ __forceinline__ const char *align16(const E *p, int &off_elems) {
 // waited on the barrier sees them.  All lanes call.
 template <class L, class T, bool ODD, bool ALIGNED, class I, int TW>
 __device__ __forceinline__ void issue_tile(const SweepArgs<typename Storage<T>::C> &a,
-                                           const TileDesc &td, unsigned char *stage, int *off,
+                                           const TileDesc &td, const TileLinks *tl, unsigned char *stage, int *off,
                                            uint64_t *bar) {
   using SL = StageLayout<L, T, TW>;
   constexpr int W = StageShape<T, TW>::kWidth;
@@ -572,11 +586,17 @@ __device__ __forceinline__ void issue_tile(const SweepArgs<typename Storage<T>::
       }
     }
   } else if (lane == L::Q) {
-    const int nrec = __popcll(td.bnd);
     int o;
-    src = align16(a.geo.rec32 + td.rb, o);
+    if (link_parallel<T>()) {
+      const int nl = tl->dense ? 0 : tl->k0 + tl->k1;     // dense tiles read them from memory
+      src = align16(a.geo.ldesc + tl->l0, o);
+      bytes = nl > 0 ? (((uint32_t)((o + nl) * (int)sizeof(uint16_t)) + 15u) & ~15u) : 0u;
+    } else {
+      const int nrec = __popcll(td.bnd);
+      src = align16(a.geo.rec32 + td.rb, o);
+      bytes = nrec > 0 ? (((uint32_t)((o + nrec) * (int)sizeof(uint32_t)) + 15u) & ~15u) : 0u;
+    }
     off[L::Q] = o;
-    bytes = nrec > 0 ? (((uint32_t)((o + nrec) * (int)sizeof(uint32_t)) + 15u) & ~15u) : 0u;
     dst = stage + SL::kRec;
   }
   const uint32_t total = __reduce_add_sync(0xffffffffu, bytes + (src2 ? 16u : 0u));
@@ -692,6 +712,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, MinBlocks<L, T, BATCH>::v
   uint64_t *bars = reinterpret_cast<uint64_t *>(wsm + SL::kBars);
   int *offs = reinterpret_cast<int *>(wsm + SL::kOffs);
 
+  const TileLinks *const links = reinterpret_cast<const TileLinks *>(tiles + n_tiles);
   const int gw = blockIdx.x * kWarpsPerBlock + warp;
   const int nw = gridDim.x * kWarpsPerBlock;
   if (lane == 0) {
@@ -702,7 +723,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, MinBlocks<L, T, BATCH>::v
   for (int s = 0; s < NS; ++s) {
     const int tile = gw + s * nw;
     if (tile < n_tiles)
-      issue_tile<L, T, ODD, ALIGNED, I, TW>(args_for<BATCH>(a, inst, tile_inst, tile), tiles[tile],
+      issue_tile<L, T, ODD, ALIGNED, I, TW>(args_for<BATCH>(a, inst, tile_inst, tile), tiles[tile], links + tile,
                                wsm + s * SL::kStage, offs + s * NO, &bars[s]);
   }
 
@@ -728,38 +749,40 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, MinBlocks<L, T, BATCH>::v
     T *const lnk = static_cast<T *>(A.geo.lnk);
     const TileDesc td = tiles[tile];
     const int y = td.yz & 0xffff, z = td.yz >> 16;
-    const unsigned char *stg = wsm + s * SL::kStage;
+    unsigned char *stg = wsm + s * SL::kStage;
     const T *st = reinterpret_cast<const T *>(stg);
     const uint32_t *rec_s = reinterpret_cast<const uint32_t *>(stg + SL::kRec) + offs[s * NO + Q];
     const int row = A.nx * (y + A.ny * z);
+    // cut links of the tile, link by link over the lanes
+    constexpr bool kLP = link_parallel<T>();
+    TileLinks tl{};
+    if constexpr (kLP) tl = links[tile];
+    const bool tile_links = tl.k0 + tl.k1 > 0;
+    C *const ex_s = reinterpret_cast<C *>(stg);
+    const uint16_t *desc = tl.dense ? A.geo.ldesc + tl.l0
+                                    : reinterpret_cast<const uint16_t *>(stg + SL::kRec) + offs[s * NO + Q];
+    auto refill = [&]() {   // stage s consumed: fill it with the tile NS rounds ahead
+      const int nt = tile + NS * nw;
+      if (nt < n_tiles)
+        issue_tile<L, T, ODD, ALIGNED, I, TW>(args_for<BATCH>(a, inst, tile_inst, nt), tiles[nt], links + nt,
+                                 wsm + s * SL::kStage, offs + s * NO, &bars[s]);
+    };
 #pragma unroll 1
     for (int j = 0; j < TW / 32; ++j) {
     const int xl = j * 32 + lane;          // position inside the tile
     const int x = td.x0 + xl;
     const int n = row + x;
     const bool solid = (td.solid >> xl) & 1ull;
+    const int nl = j == 0 ? tl.k0 : tl.k1;                   // links of this half
+    const int l0 = tl.l0 + (j == 0 ? 0 : tl.k0);
     int boff = 0;
     uint32_t bmask = 0u;
-    if ((td.bnd >> xl) & 1ull) {
+    if (!kLP && ((td.bnd >> xl) & 1ull)) {
       const uint32_t r = rec_s[__popcll(td.bnd & ((1ull << xl) - 1ull))];
       bmask = r & ((1u << kRecShift) - 1u);
       boff = td.lb + (int)(r >> kRecShift);
       asm volatile("prefetch.global.L2 [%0];" ::"l"(coef + boff));
     }
-    C g[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const int o = ALIGNED ? (ODD ? aligned_window_offset<T>(L::ex(i)) : 0) : offs[s * NO + i];
-      g[i] = Storage<T>::load(st + i * W + o + xl);
-    }
-    if (j == TW / 32 - 1) {
-      __syncwarp();   // stage s consumed: refill it with the tile NS rounds ahead
-      const int nt = tile + NS * nw;
-      if (nt < n_tiles)
-        issue_tile<L, T, ODD, ALIGNED, I, TW>(args_for<BATCH>(a, inst, tile_inst, nt), tiles[nt],
-                                 wsm + s * SL::kStage, offs + s * NO, &bars[s]);
-    }
-    if (solid) continue;
 
     // lanes on the periodic x-edges: the row windows cannot follow the wrap.  A step
     // across x = 0 lands in column nx-1 of the row shifted by (+sy, +sz), across
@@ -772,14 +795,82 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, MinBlocks<L, T, BATCH>::v
       return (I)xc + (I)A.nx * ((I)yy + (I)A.ny * zz);
     };
     const int sy = SKEW ? A.sy : 0, sz = SKEW ? A.sz : 0;
+
+    // element of population i of position xs in the stage
+    auto slot = [&](int i, int xs) {
+      return i * W + (ALIGNED ? (ODD ? aligned_window_offset<T>(DirBits<L>::ex(i)) : 0) : offs[s * NO + i]) + xs;
+    };
+    if constexpr (kLP) {
+      if (nl > 0) {
+        if (lane < nl) asm volatile("prefetch.global.L2 [%0];" ::"l"(coef + l0 + lane));
+        if constexpr (ODD) {
+          // what does not arrive with the windows goes into the stage first: values
+          // across the x-wrap, then the populations that arrive through a cut link,
+          // left in the link buffer by the previous (even) step
+          if (!ALIGNED) {
+            if (xlo && !solid) {
+#pragma unroll
+              for (int i = 0; i < Q; ++i)
+                if (L::ex(i) > 0)
+                  ex_s[slot(i, xl)] = Storage<T>::load(pop + (I)L::opp(i) * S + across(nxm1, sy - L::ey(i), sz - L::ez(i)));
+            }
+            if (xhi && !solid) {
+#pragma unroll
+              for (int i = 0; i < Q; ++i)
+                if (L::ex(i) < 0)
+                  ex_s[slot(i, xl)] = Storage<T>::load(pop + (I)L::opp(i) * S + across(0, -sy - L::ey(i), -sz - L::ez(i)));
+            }
+            __syncwarp();
+          }
+#pragma unroll 1
+          for (int k = lane; k < nl; k += 32) {
+            const int e = desc[l0 - tl.l0 + k];
+            ex_s[slot(L::opp_rt(e >> kLinkDirShift), j * 32 + (e & 31))] = Storage<T>::load(lnk + l0 + k);
+          }
+          __syncwarp();
+        }
+      }
+    }
+    C g[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const int o = ALIGNED ? (ODD ? aligned_window_offset<T>(L::ex(i)) : 0) : offs[s * NO + i];
+      g[i] = Storage<T>::load(st + i * W + o + xl);
+    }
+    if (j == TW / 32 - 1 && !tile_links) {
+      __syncwarp();
+      refill();
+    }
+    // First half of the boundary scheme (Eqs. 2.10, 2.13) with a lane per link: the part
+    // of the node's pre-collision values, read from the stage.  A lane per node runs
+    // every cut direction that any node of the warp has, a few lanes at a time; a lane per link
+    // runs once (a curved wall leaves some 16 links in a half that has any).
+    C part[kSparseLinks / 32];
+    if constexpr (kLP) {
+      if (nl > 0) {
+        auto first = [&](int k) {
+          const int e = desc[l0 - tl.l0 + k], d = e >> kLinkDirShift, xs = j * 32 + (e & 31);
+          const LinkCoef<C> c = load_coef_nc(coef + l0 + k);
+          return A.one_minus_b * ex_s[slot(L::opp_rt(d), xs)] + c.a * ex_s[slot(d, xs)];
+        };
+#pragma unroll
+        for (int r = 0; r < kSparseLinks / 32; ++r)
+          if (r * 32 + lane < nl) part[r] = first(r * 32 + lane);
+#pragma unroll 1
+        for (int k = kSparseLinks + lane; k < nl; k += 32) lnk[l0 + k] = first(k);   // free until the step writes it
+        __syncwarp();
+      }
+    }
+
+    if (!solid) {
     // (a node can be on both edges when nx = 1)
-    if (ODD && !ALIGNED && xlo) {          // aligned rows: staged with the windows
+    if (ODD && !ALIGNED && xlo && !(kLP && nl > 0)) {          // aligned rows: staged with the windows
 #pragma unroll
       for (int i = 0; i < Q; ++i)
         if (L::ex(i) > 0)
           g[i] = Storage<T>::load(pop + (I)L::opp(i) * S + across(nxm1, sy - L::ey(i), sz - L::ez(i)));
     }
-    if (ODD && !ALIGNED && xhi) {
+    if (ODD && !ALIGNED && xhi && !(kLP && nl > 0)) {
 #pragma unroll
       for (int i = 0; i < Q; ++i)
         if (L::ex(i) < 0)
@@ -869,6 +960,41 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, MinBlocks<L, T, BATCH>::v
           if (!ODD) Storage<T>::store(lnk + kk, v);          // read by the next odd step
           else Storage<T>::store(pn + (I)i * S, v);          // slot i of x_f itself
         }
+      }
+    }
+    if constexpr (kLP) {
+      if (nl > 0) {                        // hand f' to the lanes of the links
+#pragma unroll
+        for (int i = 1; i < Q; ++i) {
+          const int o = ALIGNED ? (ODD ? aligned_window_offset<T>(L::ex(i)) : 0) : offs[s * NO + i];
+          ex_s[i * W + o + xl] = gp[i];
+        }
+      }
+    }
+    }  // !solid
+
+    // second half of the boundary scheme: the part of the post-collision values
+    if constexpr (kLP) {
+      if (nl > 0) {
+        __syncwarp();
+        auto second = [&](int k, C p) {
+          const int e = desc[l0 - tl.l0 + k], d = e >> kLinkDirShift, i = L::opp_rt(d), xs = j * 32 + (e & 31);
+          const LinkCoef<C> c = load_coef_nc(coef + l0 + k);
+          const C v = p + c.bb * ex_s[slot(i, xs)] + c.c * ex_s[slot(d, xs)] + c.w * A.wfac;
+          if (!ODD) lnk[l0 + k] = v;                                   // read by the next odd step
+          else pop[(I)(row + td.x0 + xs) + (I)i * S] = v;              // slot i of x_f itself
+        };
+#pragma unroll
+        for (int r = 0; r < kSparseLinks / 32; ++r)
+          if (r * 32 + lane < nl) second(r * 32 + lane, part[r]);
+#pragma unroll 1
+        for (int k = kSparseLinks + lane; k < nl; k += 32) second(k, lnk[l0 + k]);
+      }
+      if (j == TW / 32 - 1 && tile_links) {
+        // the stage was written by these lanes: order that before the bulk copies
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        refill();
       }
     }
     }

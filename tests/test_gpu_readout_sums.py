@@ -36,7 +36,9 @@ def test_readout_sums_match_fp64(lattice, precision, rho0):
     scale = {"f64": 1e-3, "f32": 1e-3, "f16": 1.0}[precision]
     wr = lat.w[:, None] * rho0
     f = wr + scale * g
-    held = f - wr                                     # what the context is given
+    # what the context stores: f - w rho0 in one rounding (a fused multiply-add), then the type's
+    wide = np.longdouble
+    held = (f.astype(wide) - lat.w[:, None].astype(wide) * wide(rho0)).astype(np.float64)
     t = {"f64": np.float64, "f32": np.float32, "f16": np.float16}[precision]
     with np.errstate(over="ignore"):
         held = held.astype(t).astype(np.float64)
