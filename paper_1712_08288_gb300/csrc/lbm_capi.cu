@@ -227,17 +227,7 @@ static void refresh_args(lbm_ctx *c) {
     a.wfac = C(wall_factor(c, c->t));
     a.status = c->status;
     a.wait_polls = c->wait_polls;
-    with_lat(c->lattice, [&](auto lat) {
-      using L = decltype(lat);
-      const long long S = slot_stride(c->N), nxl = c->nx, nxy = (long long)c->nx * c->ny;
-      for (int i = 0; i < 19; ++i) a.koff_even[i] = a.koff_odd[i] = 0;
-      for (int i = 0; i < L::Q; ++i) {
-        a.koff_even[i] = L::opp(i) * S;
-        a.koff_odd[i] = i * S + L::ex(i) + nxl * L::ey(i) + nxy * L::ez(i);
-      }
-      a.kwrap = nxl * (1 + c->sy) + nxy * c->sz;
-      return 0;
-    });
+    for (int i = 0; i < 19; ++i) a.kslot[i] = i * slot_stride(c->N);
   };
   fill(c->a64);
   fill(c->a32);

@@ -139,14 +139,7 @@ struct SweepArgs : FixedPart<C> {
   C wfac;                    // factor on every link's wall velocity in this step
   int *status;               // bit 0: non-finite density seen, bit 1: bounded wait gave up
   int wait_polls;            // polls of a tile's barrier before the sweep gives up
-  // element offsets of the stores of an interior node: even step slot opp(i) of
-  // the node itself, odd step slot i of x + e_i (no wrap)
-  long long koff_even[19];
-  long long koff_odd[19];
-  // the odd-step store of node (0, y, z) across the x-wrap lands at koff_odd[i] +
-  // kwrap, that of node (nx-1, y, z) at koff_odd[i] - kwrap, when the skew-shifted
-  // rows stay inside the grid: kwrap = nx (1 + sy) + nx ny sz
-  long long kwrap;
+  long long kslot[19];       // first element of slot i: i S
   // when non-null, the sweep also writes every fluid node's pre-collision
   // deviations g_i(x, t) here, natural layout save[i*N + n] (adjoint recomputation)
   C *save = nullptr;

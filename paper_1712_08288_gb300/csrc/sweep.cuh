@@ -893,58 +893,42 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, MinBlocks<L, T, BATCH>::v
     C gp[Q];
     if (collide<L, C, T>(g, gp, A)) atomicOr(A.status, 1);
 
-    T *const pn = pop + n;
+    // start of slot i: a constant operand for a single context, arithmetic for a batch
+    // (whose arguments sit in memory)
+    auto slot0 = [&](int i) -> I { return BATCH ? (I)i * S : (I)A.kslot[i]; };
     if (!ODD) {
 #pragma unroll
-      for (int i = 0; i < Q; ++i) Storage<T>::store(pn + (I)A.koff_even[i], gp[i]);   // slot opp(i) of x
+      for (int i = 0; i < Q; ++i) Storage<T>::store(pop + (slot0(L::opp(i)) + (I)n), gp[i]);   // slot opp(i) of x
     } else {
-      // rows y +- 1, z +- 1 stay inside the grid for the whole tile: constant offsets
-      const bool rows_inside =
-          y > 0 && y < A.ny - 1 && (L::D == 2 || (z > 0 && z < A.nz - 1));
-      if (rows_inside) {
+      // slot i of x + e_i = column X + row Y + plane Z, each wrapped by itself: a handful
+      // of selections per node and the same instructions for every node, instead of
+      // separate code for interior rows, wrapped rows and the x-edges (whose
+      // instruction fetches cost the FP64 odd step a fifth of its time).
+      const I nx = (I)A.nx, nxy = (I)A.nx * A.ny;
+      const I X[3] = {(I)(xlo ? nxm1 : x - 1), (I)x, (I)(xhi ? 0 : x + 1)};
+      I Y[3][3], Z[3][3];      // [e_x + 1][e + 1]: a skewed wrap shifts the rows across it
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-          const int ex = L::ex(i);
-          if ((ex > 0 && xhi) || (ex < 0 && xlo)) continue;   // crosses the x-wrap
-          Storage<T>::store(pn + (I)A.koff_odd[i], gp[i]);     // slot i of x + e_i
+      for (int e = 0; e < 3; ++e) {
+        int ys = y, zs = z;
+        if (SKEW && e == 0 && xlo) {
+          ys = wrap1(ys + sy, A.ny);
+          zs = wrap1(zs + sz, A.nz);
         }
-        // stores across the periodic x-wrap: when the skew-shifted rows (y +- sy +
-        // e_y, z +- sz + e_z) stay inside the grid, the target is the regular odd-step
-        // offset moved by +-kwrap; otherwise every row index is wrapped
-        if (xlo) {
-          const int ys = y + sy, zs = z + sz;
-          if (ys >= 1 && ys <= A.ny - 2 && (L::D == 2 || (zs >= 1 && zs <= A.nz - 2))) {
-#pragma unroll
-            for (int i = 0; i < Q; ++i)
-              if (L::ex(i) < 0) Storage<T>::store(pn + (I)(A.koff_odd[i] + A.kwrap), gp[i]);
-          } else {
-#pragma unroll
-            for (int i = 0; i < Q; ++i)
-              if (L::ex(i) < 0)
-                Storage<T>::store(pop + (I)i * S + across(nxm1, sy + L::ey(i), sz + L::ez(i)), gp[i]);
-          }
+        if (SKEW && e == 2 && xhi) {
+          ys = wrap1(ys - sy, A.ny);
+          zs = wrap1(zs - sz, A.nz);
         }
-        if (xhi) {
-          const int ys = y - sy, zs = z - sz;
-          if (ys >= 1 && ys <= A.ny - 2 && (L::D == 2 || (zs >= 1 && zs <= A.nz - 2))) {
+        Y[e][0] = nx * (ys == 0 ? A.ny - 1 : ys - 1);
+        Y[e][1] = nx * ys;
+        Y[e][2] = nx * (ys == A.ny - 1 ? 0 : ys + 1);
+        Z[e][0] = L::D == 3 ? nxy * (zs == 0 ? A.nz - 1 : zs - 1) : I(0);
+        Z[e][1] = L::D == 3 ? nxy * zs : I(0);
+        Z[e][2] = L::D == 3 ? nxy * (zs == A.nz - 1 ? 0 : zs + 1) : I(0);
+      }
 #pragma unroll
-            for (int i = 0; i < Q; ++i)
-              if (L::ex(i) > 0) Storage<T>::store(pn + (I)(A.koff_odd[i] - A.kwrap), gp[i]);
-          } else {
-#pragma unroll
-            for (int i = 0; i < Q; ++i)
-              if (L::ex(i) > 0)
-                Storage<T>::store(pop + (I)i * S + across(0, -sy + L::ey(i), -sz + L::ez(i)), gp[i]);
-          }
-        }
-      } else {
-        // rows of the tile touch a periodic edge in y or z: wrap every neighbour
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-          const long long dn = wrap_index(x, y, z, L::ex(i), L::ey(i), L::ez(i), A.nx, A.ny, A.nz,
-                                          A.sy, A.sz);
-          Storage<T>::store(pop + (I)i * S + (I)dn, gp[i]);
-        }
+      for (int i = 0; i < Q; ++i) {
+        const int ex = L::ex(i) + 1, ey = L::ey(i) + 1, ez = L::ez(i) + 1;
+        Storage<T>::store(pop + (X[ex] + (Y[ex][ey] + Z[ex][ez]) + slot0(i)), gp[i]);
       }
     }
 
@@ -958,7 +942,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, MinBlocks<L, T, BATCH>::v
           const int i = L::opp(dd);
           const C v = A.one_minus_b * g[i] + c.a * g[dd] + c.bb * gp[i] + c.c * gp[dd] + c.w * A.wfac;
           if (!ODD) Storage<T>::store(lnk + kk, v);          // read by the next odd step
-          else Storage<T>::store(pn + (I)i * S, v);          // slot i of x_f itself
+          else Storage<T>::store(pop + ((I)i * S + (I)n), v);  // slot i of x_f itself
         }
       }
     }
