@@ -242,9 +242,11 @@ int lbm_set_link_values(lbm_ctx *ctx, const double *q, const double *uw);
  * exactly what lbm_step computes), for the loss
  *   J = sum over fluid nodes n with mask[n] != 0 of |u(x_n, T) - u_target(x_n)|^2,
  * u the reported velocity after the n_steps (T = current time + n_steps).
- * The forward run keeps a raw checkpoint every checkpoint_every steps (0 = about
+ * The forward run keeps a checkpoint every checkpoint_every steps (0 = every state of
+ * the run where they take at most 4 GiB and 1/16 of the free memory, else about
  * sqrt(n_steps)); the backward pass recomputes one segment at a time from its
- * checkpoint and runs the adjoint sweep through it.  On return the context is in
+ * checkpoint and runs the adjoint sweep through it.  The last segment, or the only
+ * one, keeps its states and is not recomputed.  On return the context is in
  * the state after the forward run (as if lbm_step(n_steps) had been called).
  *   mask      nodes bytes (host); u_target D*nodes doubles (host, node-major).
  *   loss      J (may be NULL).

@@ -24,6 +24,7 @@
 //     (meq_adjoint); lambda(t) = M^T nu + boundary terms, and
 //     dJ/ds_k += mu_k * (-(m_k - meq_k)).
 // Adjoint entries of solid nodes are zero and stay zero (never written).
+#include "node_sums.cuh"
 #include "sweep.cuh"
 
 namespace lbm {
@@ -42,11 +43,13 @@ template <class L, class T, class C>
 __global__ void export_state_kernel(AuxArgs a, bool odd, C *out) {
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < a.N;
        n += (long long)gridDim.x * blockDim.x) {
-    const bool solid = a.cls[n] == kSolid;
+    const int cls = a.cls[n];
+    C g[L::Q];
 #pragma unroll
-    for (int i = 0; i < L::Q; ++i)
-      out[(long long)i * a.N + n] =
-          solid ? C(0) : C(Storage<T>::load(population_address<L, T>(i, n, odd, a)));
+    for (int i = 0; i < L::Q; ++i) g[i] = C(0);
+    if (cls != kSolid) load_node<L, T>(g, (int)n, cls, odd, a);
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) out[(long long)i * a.N + n] = g[i];
   }
 }
 
@@ -62,38 +65,67 @@ __global__ void import_state_kernel(AuxArgs a, const C *in) {
   }
 }
 
-// J and lambda(T); u = j/rho0 + g/2 from the natural-layout deviations
-template <class L, class C>
-__global__ void loss_kernel(AuxArgs a, const C *g, const uint8_t *mask, const double *u_target,
-                            C *lam, double *J) {
+// J and lambda(T) from the state in the AA layout: lambda_i = 2 (u - u*).e_i / rho0 on
+// masked fluid nodes, zero elsewhere (where only the zeros are written: FP64 arithmetic
+// is what this kernel would otherwise spend its time on).
+template <class L, class T>
+__global__ void loss_kernel(AuxArgs a, bool odd, const uint8_t *mask, const double *u_target,
+                            typename Storage<T>::C *lam, double *J) {
+  using C = typename Storage<T>::C;
   double acc = 0.0;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < a.N;
        n += (long long)gridDim.x * blockDim.x) {
-    const bool on = a.cls[n] != kSolid && mask[n];
-    double j[3] = {0.0, 0.0, 0.0};
-    if (on) {
+    const int cls = mask[n] ? (int)a.cls[n] : (int)kSolid;
+    C v[3] = {C(0), C(0), C(0)}, vxy[2] = {C(0), C(0)}, vxz[2] = {C(0), C(0)}, vyz[2] = {C(0), C(0)};
+    C vc[4] = {C(0), C(0), C(0), C(0)};
+    if (cls != kSolid) {
+      C g[L::Q];
+      load_node<L, T>(g, (int)n, cls, odd, a);
+      double drho, j[3], d[3] = {0.0, 0.0, 0.0};
+      node_sums<L>(g, drho, j);
 #pragma unroll
-      for (int i = 0; i < L::Q; ++i) {
-        const double v = (double)g[(long long)i * a.N + n];
-        j[0] += L::ex(i) * v;
-        j[1] += L::ey(i) * v;
-        j[2] += L::ez(i) * v;
+      for (int k = 0; k < L::D; ++k) {
+        const double diff = velocity(j[k], a, k) - u_target[n * L::D + k];
+        acc += diff * diff;
+        d[k] = 2.0 / a.rho0 * diff;
+        v[k] = C(d[k]);
+      }
+      // e_i . d for one direction of each pair (the other has the opposite sign)
+      const double p = d[0] + d[1], m = d[0] - d[1];
+      if (L::Q != 15) {
+        vxy[0] = C(p);
+        vxy[1] = C(m);
+      }
+      if (L::Q == 19) {
+        vxz[0] = C(d[0] + d[2]);
+        vxz[1] = C(d[0] - d[2]);
+        vyz[0] = C(d[1] + d[2]);
+        vyz[1] = C(d[1] - d[2]);
+      }
+      if (L::Q == 15) {
+        vc[0] = C(p + d[2]);
+        vc[1] = C(p - d[2]);
+        vc[2] = C(m + d[2]);
+        vc[3] = C(m - d[2]);
       }
     }
-    double diff[3] = {0.0, 0.0, 0.0};
-    if (on)
-      for (int k = 0; k < L::D; ++k) {
-        diff[k] = j[k] / a.rho0 + 0.5 * a.g[k] - u_target[n * L::D + k];
-        acc += diff[k] * diff[k];
-      }
+    if (!lam) continue;
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
-      const double v = 2.0 / a.rho0 * (L::ex(i) * diff[0] + L::ey(i) * diff[1] + L::ez(i) * diff[2]);
-      lam[(long long)i * a.N + n] = C(v);
+      const int ex = L::ex(i), ey = L::ey(i), ez = L::ez(i);
+      C w = C(0);
+      if (ex && ey && ez) w = (ex * ey > 0 ? (ex * ez > 0 ? vc[0] : vc[1]) : (ex * ez > 0 ? vc[2] : vc[3])) * C(ex);
+      else if (ex && ey) w = (ex * ey > 0 ? vxy[0] : vxy[1]) * C(ex);
+      else if (ex && ez) w = (ex * ez > 0 ? vxz[0] : vxz[1]) * C(ex);
+      else if (ey && ez) w = (ey * ez > 0 ? vyz[0] : vyz[1]) * C(ey);
+      else if (ex) w = v[0] * C(ex);
+      else if (ey) w = v[1] * C(ey);
+      else if (ez) w = v[2] * C(ez);
+      lam[(long long)i * a.N + n] = w;
     }
   }
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) atomic_add_double(J, acc);
+  if ((threadIdx.x & 31) == 0 && acc != 0.0) atomic_add_double(J, acc);
 }
 
 // Link data of the adjoint step.  The gradients with respect to a link's wall
@@ -451,18 +483,16 @@ cudaError_t launch_import_state(int lattice, int precision, const AuxArgs &a, co
   });
 }
 
-cudaError_t launch_loss(int lattice, int precision, const AuxArgs &a, const void *g,
-                        const uint8_t *mask, const double *u_target, void *lam, double *J,
-                        cudaStream_t st) {
+cudaError_t launch_loss(int lattice, int precision, const AuxArgs &a, bool odd, const uint8_t *mask,
+                        const double *u_target, void *lam, double *J, cudaStream_t st) {
   return with_lattice(lattice, [&](auto lat) {
     using L = decltype(lat);
-    if (precision == 0)
-      loss_kernel<L, double><<<adj_blocks(a.N), 256, 0, st>>>(a, static_cast<const double *>(g), mask,
-                                                              u_target, static_cast<double *>(lam), J);
-    else
-      loss_kernel<L, float><<<adj_blocks(a.N), 256, 0, st>>>(a, static_cast<const float *>(g), mask,
-                                                             u_target, static_cast<float *>(lam), J);
-    return cudaGetLastError();
+    return with_storage(precision, [&](auto *tp) {
+      using T = std::remove_pointer_t<decltype(tp)>;
+      using C = typename Storage<T>::C;
+      loss_kernel<L, T><<<adj_blocks(a.N), 256, 0, st>>>(a, odd, mask, u_target, static_cast<C *>(lam), J);
+      return cudaGetLastError();
+    });
   });
 }
 

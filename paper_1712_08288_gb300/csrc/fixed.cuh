@@ -147,34 +147,29 @@ struct FxQuad {
   }
 };
 
-// Change of the populations by the relaxed rows, t = M^T r with r_k = s_k (m_k - m^eq_k)
-// / |M_k|^2, and by the force (r = -F on the momentum rows), from the deviations v.  The
-// equilibrium is folded into the moment sums in closed form (meq() in sweep.cuh); the
-// constant of a row carries the factor taken out of its sum (fx_row_scale).  Rows
+// Momentum and relaxed moments of the deviations v: n_k = (m_k - m^eq_k) / fx_neq_scale, the
+// equilibrium folded into the moment sums in closed form (meq() in sweep.cuh).  Rows
 // whose rate can exceed 1/4 are doubled in the sum.
-LBM_HD void fx_change(D2Q9, const i64 (&v)[9], i64 (&t)[9], i64 Fx, i64 Fy, i64 Fz, int E,
-                      const FixedArgs &fx) {
-  i64 r[9];
+template <int D>
+struct FxMomentum {
+  i64 x, y, z;
+};
+LBM_HD FxMomentum<2> fx_neq(D2Q9, const i64 (&v)[9], i64 (&n)[9], int E, const FixedArgs &fx) {
   const i64 s0 = v[1] + v[3], s1 = v[2] + v[4], s2 = v[5] + v[7], s3 = v[6] + v[8];
   const i64 d0 = v[1] - v[3], d1 = v[2] - v[4], d2 = v[5] - v[7], d3 = v[6] - v[8];
   const i64 F = s0 + s1, K = s2 + s3;
   const i64 jx = d0 + d2 - d3, jy = d1 + d2 + d3;
   const FxQuad<2> q(jx, jy, 0, E, fx);
   const i64 j2 = q.xx + q.yy;
-  r[1] = fx_mul(2 * K + ((F - 2 * v[0] - 3 * j2) >> 1), fx.row[1]);
-  r[2] = fx_mul(v[0] - F + j2, fx.row[2]);
-  r[4] = fx_mul(2 * jx - 3 * d0, fx.row[4]);
-  r[6] = fx_mul(2 * jy - 3 * d1, fx.row[6]);
-  r[7] = fx_mul((s0 - s1 - q.xx + q.yy) << 1, fx.row[7]);
-  r[8] = fx_mul((s2 - s3 - q.xy) << 1, fx.row[8]);
-  r[0] = 0;
-  r[3] = -Fx;
-  r[5] = -Fy;
-  fmt<false, i64>(D2Q9{}, r, t);
+  n[1] = 2 * K + ((F - 2 * v[0] - 3 * j2) >> 1);
+  n[2] = v[0] - F + j2;
+  n[4] = 2 * jx - 3 * d0;
+  n[6] = 2 * jy - 3 * d1;
+  n[7] = (s0 - s1 - q.xx + q.yy) << 1;
+  n[8] = (s2 - s3 - q.xy) << 1;
+  return {jx, jy, 0};
 }
-LBM_HD void fx_change(D3Q15, const i64 (&v)[15], i64 (&t)[15], i64 Fx, i64 Fy, i64 Fz, int E,
-                      const FixedArgs &fx) {
-  i64 r[15];
+LBM_HD FxMomentum<3> fx_neq(D3Q15, const i64 (&v)[15], i64 (&n)[15], int E, const FixedArgs &fx) {
   const i64 s0 = v[1] + v[2], s1 = v[3] + v[4], s2 = v[5] + v[6];
   const i64 d0 = v[1] - v[2], d1 = v[3] - v[4], d2 = v[5] - v[6];
   const i64 s3 = v[7] + v[14], s4 = v[8] + v[13], s5 = v[9] + v[12], s6 = v[10] + v[11];
@@ -185,25 +180,20 @@ LBM_HD void fx_change(D3Q15, const i64 (&v)[15], i64 (&t)[15], i64 Fx, i64 Fy, i
   const i64 jx = d0 + cg - ch, jy = d1 + cg + ch, jz = d2 + ce + cf;
   const FxQuad<3> q(jx, jy, jz, E, fx);
   const i64 j2 = q.xx + q.yy + q.zz;
-  r[1] = fx_mul(2 * K - v[0] - j2, fx.row[1]);
-  r[2] = fx_mul(3 * v[0] - F + j2, fx.row[2]);
-  r[4] = fx_mul(2 * jx - 3 * d0, fx.row[4]);
-  r[6] = fx_mul(2 * jy - 3 * d1, fx.row[6]);
-  r[8] = fx_mul(2 * jz - 3 * d2, fx.row[8]);
-  r[9] = fx_mul(2 * (s0 - q.xx) - s1 - s2 + q.yy + q.zz, fx.row[9]);
-  r[10] = fx_mul((s1 - s2 - q.yy + q.zz) << 1, fx.row[10]);
-  r[11] = fx_mul(ca - cb - q.xy, fx.row[11]);
-  r[12] = fx_mul(cc + cd - q.yz, fx.row[12]);
-  r[13] = fx_mul(cc - cd - q.xz, fx.row[13]);
-  r[14] = fx_mul(ce - cf, fx.row[14]);
-  r[0] = 0;
-  r[3] = -Fx;
-  r[5] = -Fy;
-  r[7] = -Fz;
-  fmt<false, i64>(D3Q15{}, r, t);
+  n[1] = 2 * K - v[0] - j2;
+  n[2] = 3 * v[0] - F + j2;
+  n[4] = 2 * jx - 3 * d0;
+  n[6] = 2 * jy - 3 * d1;
+  n[8] = 2 * jz - 3 * d2;
+  n[9] = 2 * (s0 - q.xx) - s1 - s2 + q.yy + q.zz;
+  n[10] = (s1 - s2 - q.yy + q.zz) << 1;
+  n[11] = ca - cb - q.xy;
+  n[12] = cc + cd - q.yz;
+  n[13] = cc - cd - q.xz;
+  n[14] = ce - cf;
+  return {jx, jy, jz};
 }
-LBM_HD void fx_change(D3Q19, const i64 (&v)[19], i64 (&t)[19], i64 Fx, i64 Fy, i64 Fz, int E,
-                      const FixedArgs &fx) {
+LBM_HD FxMomentum<3> fx_neq(D3Q19, const i64 (&v)[19], i64 (&n)[19], int E, const FixedArgs &fx) {
   i64 s[9], d[9];
 #ifdef __CUDA_ARCH__
 #pragma unroll
@@ -220,50 +210,89 @@ LBM_HD void fx_change(D3Q19, const i64 (&v)[19], i64 (&t)[19], i64 Fx, i64 Fy, i
   const i64 jz = d[2] + d[5] - d[6] + d[7] - d[8];
   const FxQuad<3> q(jx, jy, jz, E, fx);
   const i64 j2 = q.xx + q.yy + q.zz, pw = q.yy - q.zz, px = 2 * q.xx - q.yy - q.zz;
-  // Rows e and eps act through one value per face, edge and the rest node, with factors
-  // up to 30 on their rates: they are taken 8 and 4 times larger, rounded where they are
-  // used, and the rest node gets what keeps the sum over all nodes zero.  (The
-  // sum of row eps, up to 178 g, is taken in units 4 times larger.)
-  const i64 r1 = fx_mul(K - v[0] - j2, fx.row[1]);
-  const i64 r2 = fx_mul(9 * (v[0] >> 2) - 7 * (F >> 2) - 2 * (K >> 2) + 11 * (j2 >> 3), fx.row[2]);
-  const i64 Ce = r1 + ((r2 + 2) >> 2), Cf = -((11 * r1 + 4) >> 3) - r2;
-  const i64 rx = fx_mul(jx - 3 * d[0], fx.row[4]), ry = fx_mul(jy - 3 * d[1], fx.row[6]);
-  const i64 rz = fx_mul(jz - 3 * d[2], fx.row[8]);
-  const i64 r9 = fx_mul(2 * s[0] - s[1] - s[2] + Exyz - px, fx.row[9]);
-  const i64 r10 = fx_mul(2 * (s[1] + s[2] - 2 * s[0]) + Exyz + (px >> 1), fx.row[10]);
-  const i64 r11 = fx_mul(s[1] - s[2] + Ey - pw, fx.row[11]);
-  const i64 r12 = fx_mul(2 * (s[2] - s[1]) + Ey + (pw >> 1), fx.row[12]);
-  const i64 r13 = fx_mul((s[3] - s[4] - q.xy) << 1, fx.row[13]);
-  const i64 r14 = fx_mul((s[7] - s[8] - q.yz) << 1, fx.row[14]);
-  const i64 r15 = fx_mul((s[5] - s[6] - q.xz) << 1, fx.row[15]);
-  const i64 r16 = fx_mul(d[3] + d[4] - d[5] - d[6], fx.row[16]);
-  const i64 r17 = fx_mul(d[4] - d[3] + d[7] + d[8], fx.row[17]);
-  const i64 r18 = fx_mul(d[5] - d[6] - d[7] + d[8], fx.row[18]);
-  // back-transform (fmt() in moments.cuh)
-  const i64 A = r9 + r10, B = r11 + r12;
-  const i64 Y = Cf - r9 + 2 * r10, Z = r11 - 2 * r12;
+  n[1] = K - v[0] - j2;
+  n[2] = 9 * (v[0] >> 2) - 7 * (F >> 2) - 2 * (K >> 2) + 11 * (j2 >> 3);   // up to 178 g: a quarter of it
+  n[4] = jx - 3 * d[0];
+  n[6] = jy - 3 * d[1];
+  n[8] = jz - 3 * d[2];
+  n[9] = 2 * s[0] - s[1] - s[2] + Exyz - px;
+  n[10] = 2 * (s[1] + s[2] - 2 * s[0]) + Exyz + (px >> 1);
+  n[11] = s[1] - s[2] + Ey - pw;
+  n[12] = 2 * (s[2] - s[1]) + Ey + (pw >> 1);
+  n[13] = (s[3] - s[4] - q.xy) << 1;
+  n[14] = (s[7] - s[8] - q.yz) << 1;
+  n[15] = (s[5] - s[6] - q.xz) << 1;
+  n[16] = d[3] + d[4] - d[5] - d[6];
+  n[17] = d[4] - d[3] + d[7] + d[8];
+  n[18] = d[5] - d[6] - d[7] + d[8];
+  return {jx, jy, jz};
+}
+// (m_k - m^eq_k) / n_k, 0 for the conserved rows
+template <class L>
+LBM_HD constexpr double fx_neq_scale(int k) {
+  if (L::conserved(k)) return 0.0;
+  if (L::Q == 9) return k == 1 ? 2.0 : (k == 2 ? 3.0 : (k >= 7 ? 0.5 : 1.0));
+  if (L::Q == 15) return k == 2 ? 5.0 : (k == 4 || k == 6 || k == 8 ? 5.0 / 3 : (k == 10 ? 0.5 : 1.0));
+  return k == 1 ? 19.0 : (k == 2 ? 4.0 : (k == 4 || k == 6 || k == 8 ? 5.0 / 3 : (k >= 13 && k <= 15 ? 0.5 : 1.0)));
+}
+
+// Rows e and eps of D3Q19 act through one value per face, edge and the rest node, with
+// factors up to 30 on their rates: they are taken 8 and 4 times larger and rounded where
+// they are used.
+template <class L>
+LBM_HD constexpr int fx_fine(int k) { return L::Q == 19 ? (k == 1 ? 3 : (k == 2 ? 2 : 0)) : 0; }
+
+// Change of the populations by the relaxed rows, t = M^T r with r_k = s_k (m_k - m^eq_k)
+// / |M_k|^2, and by the force (r = -F on the momentum rows), from the deviations v.
+template <class L>
+LBM_HD void fx_change(L, const i64 (&v)[L::Q], i64 (&t)[L::Q], i64 Fx, i64 Fy, i64 Fz, int E,
+                      const FixedArgs &fx) {
+  i64 n[L::Q], r[L::Q];
+  fx_neq(L{}, v, n, E, fx);
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int k = 0; k < L::Q; ++k) r[k] = L::conserved(k) ? 0 : fx_mul(n[k], fx.row[k]);
+  r[3] = -Fx;
+  r[5] = -Fy;
+  if (L::D == 3) r[7] = -Fz;
+  fmt<false, i64>(L{}, r, t);
+}
+LBM_HD void fx_change(D3Q19, const i64 (&v)[19], i64 (&t)[19], i64 Fx, i64 Fy, i64 Fz, int E,
+                      const FixedArgs &fx) {
+  i64 n[19], r[19];
+  fx_neq(D3Q19{}, v, n, E, fx);
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int k = 0; k < 19; ++k) r[k] = D3Q19::conserved(k) ? 0 : fx_mul(n[k], fx.row[k]);
+  // the back-transform (fmt() in moments.cuh); the rest node gets what keeps the sum over all
+  // nodes zero
+  const i64 Ce = r[1] + ((r[2] + 2) >> 2), Cf = -((11 * r[1] + 4) >> 3) - r[2];
+  const i64 A = r[9] + r[10], B = r[11] + r[12];
+  const i64 Y = Cf - r[9] + 2 * r[10], Z = r[11] - 2 * r[12];
   const i64 Pxy = Ce + A + B, Pxz = Ce + A - B, Pyz = Ce - 2 * A;
   i64 ev[9], od[9];
-  ev[0] = Cf + 2 * r9 - 4 * r10;
+  ev[0] = Cf + 2 * r[9] - 4 * r[10];
   ev[1] = Y + Z;
   ev[2] = Y - Z;
-  ev[3] = Pxy + r13;
-  ev[4] = Pxy - r13;
-  ev[5] = Pxz + r15;
-  ev[6] = Pxz - r15;
-  ev[7] = Pyz + r14;
-  ev[8] = Pyz - r14;
-  od[0] = -Fx - 4 * rx;
-  od[1] = -Fy - 4 * ry;
-  od[2] = -Fz - 4 * rz;
-  const i64 xf = rx - Fx, yf = ry - Fy, zf = rz - Fz;
-  const i64 xa = xf + r16, ya = yf - r17;
+  ev[3] = Pxy + r[13];
+  ev[4] = Pxy - r[13];
+  ev[5] = Pxz + r[15];
+  ev[6] = Pxz - r[15];
+  ev[7] = Pyz + r[14];
+  ev[8] = Pyz - r[14];
+  od[0] = -Fx - 4 * r[4];
+  od[1] = -Fy - 4 * r[6];
+  od[2] = -Fz - 4 * r[8];
+  const i64 xf = r[4] - Fx, yf = r[6] - Fy, zf = r[8] - Fz;
+  const i64 xa = xf + r[16], ya = yf - r[17];
   od[3] = xa + ya;
   od[4] = xa - ya;
-  const i64 xb = xf - r16, zb = zf + r18;
+  const i64 xb = xf - r[16], zb = zf + r[18];
   od[5] = xb + zb;
   od[6] = xb - zb;
-  const i64 yc = yf + r17, zc = zf - r18;
+  const i64 yc = yf + r[17], zc = zf - r[18];
   od[7] = yc + zc;
   od[8] = yc - zc;
   t[0] = -6 * Cf - 12 * Ce;
@@ -276,20 +305,6 @@ LBM_HD void fx_change(D3Q19, const i64 (&v)[19], i64 (&t)[19], i64 Fx, i64 Fy, i
   }
 }
 
-// factor of row k's constant relative to s_k / |M_k|^2 in fx_change (0: not used)
-inline double fx_row_scale(int lattice, int k) {
-  if (lattice == D2Q9::kLattice) {
-    const double t[9] = {0, 2, 3, 0, 1, 0, 1, 0.5, 0.5};
-    return t[k];
-  }
-  if (lattice == D3Q15::kLattice) {
-    const double t[15] = {0, 1, 5, 0, 5.0 / 3, 0, 5.0 / 3, 0, 5.0 / 3, 1, 0.5, 1, 1, 1, 1};
-    return t[k];
-  }
-  const double t[19] = {0, 8 * 19, 16, 0, 5.0 / 3, 0, 5.0 / 3, 0, 5.0 / 3, 1, 1, 1, 1, 0.5, 0.5, 0.5, 1, 1, 1};
-  return t[k];
-}
-
 inline FixedCoef fx_coef(double c) {   // c in [0, 1/4]
   const i64 b = (i64)llrint(ldexp(c, 64));
   const int lo = (int)(unsigned)b;
@@ -299,7 +314,7 @@ template <class L>
 inline FixedArgs fx_args(const double *s, double rho0, const double *F) {
   FixedArgs fx{};
   for (int k = 0; k < L::Q; ++k)
-    if (!L::conserved(k)) fx.row[k] = fx_coef(fx_row_scale(L::kLattice, k) * s[k] / row_norm2<L>(k));
+    if (!L::conserved(k)) fx.row[k] = fx_coef(ldexp(fx_neq_scale<L>(k), fx_fine<L>(k)) * s[k] / row_norm2<L>(k));
   int er = 0;
   double mr = frexp(1.0 / rho0, &er);    // [1/2, 1)
   if (mr == 0.5) {

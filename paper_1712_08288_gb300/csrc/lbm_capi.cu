@@ -418,7 +418,8 @@ static int upload_tiles(lbm_ctx *c, const uint8_t *solid, const std::vector<uint
   std::vector<uint32_t> rec32;
   std::vector<uint16_t> ldesc;
   if (bmask) rec32.reserve(bmask->size());
-  ldesc.reserve((size_t)c->n_links);
+  const bool per_link = c->precision == LBM_F64;    // the sweep's link-parallel boundary
+  if (per_link) ldesc.reserve((size_t)c->n_links);
   int rb = 0;
   for (int z = 0; z < c->nz; ++z)
     for (int y = 0; y < c->ny; ++y)
@@ -440,8 +441,8 @@ static int upload_tiles(lbm_ctx *c, const uint8_t *solid, const std::vector<uint
             const uint32_t m = (*bmask)[rb], off = (uint32_t)(*boff)[rb];
             if (!d.bnd) d.lb = d.l0 = (int)off;
             (k < 32 ? d.k0 : d.k1) += (unsigned short)__builtin_popcount(m);
-            for (int dir = 1; dir < c->Q; ++dir)
-              if ((m >> dir) & 1u) ldesc.push_back((uint16_t)((k & 31) | (dir << kLinkDirShift)));
+            for (uint32_t w = per_link ? m : 0u; w != 0; w &= w - 1)
+              ldesc.push_back((uint16_t)((k & 31) | (__builtin_ctz(w) << kLinkDirShift)));
             d.bnd |= 1ull << k;
             rec32.push_back(m | ((off - (uint32_t)d.lb) << kRecShift));
             ++rb;
@@ -993,6 +994,21 @@ namespace {
 // workspace slots (lbm_ctx::adj_ws)
 enum AdjSlot { kCk = 0, kSeg, kFin, kLam0, kLam1, kMask, kUt, kGs, kTot, kAcc, kDcoef, kJ, kGpart };
 
+// Whether a run of T steps keeps every state instead of checkpoints (checkpoint_every =
+// 0).  The forward sweep then writes each state once (half a step's traffic more) and the
+// backward pass recomputes nothing (a whole step's traffic less, and a launch).  Limits:
+// 4 GiB in all -- sqrt(T) checkpoints of a run of that length take up to a few GiB
+// themselves -- and, where the workspace has to grow for it, 1/16 of the free memory.
+// D3Q19 FP32, 64^3 x 144 steps (2.9 GB), forward and backward: 6.7 -> 4.8 ms.
+constexpr size_t kKeepAllBytes = (size_t)4 << 30;
+bool keep_every_state(const lbm_ctx *c, long long T, size_t state) {
+  if (state == 0 || (size_t)T > kKeepAllBytes / state) return false;
+  const size_t all = state * (size_t)T, have = c->adj_ws[kSeg].second;
+  if (have >= all) return true;
+  size_t free_b = 0, total_b = 0;
+  return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && all - have <= free_b / 16;
+}
+
 int adjoint_forward_impl(lbm_ctx *c, int n_steps, int checkpoint_every, const uint8_t *mask,
                          const double *u_target, double *loss) {
   c->tape.valid = false;
@@ -1003,12 +1019,12 @@ int adjoint_forward_impl(lbm_ctx *c, int n_steps, int checkpoint_every, const ui
     return fail(c, LBM_ESTATE, "lbm_adjoint: differentiates the single-node scheme; two-node is on");
   if (!c->geometry_set) return fail(c, LBM_ESTATE, "lbm_adjoint: geometry not set");
   const long long T = n_steps;
-  long long K = checkpoint_every;
-  if (K == 0) K = (long long)std::ceil(std::sqrt((double)T));
-  if (K > T) K = T;
-  const long long nseg = (T + K - 1) / K;
   const size_t csize = c->precision == LBM_F64 ? sizeof(double) : sizeof(float);
   const size_t state = (size_t)c->Q * c->N * csize;               // natural layout, compute type
+  long long K = checkpoint_every;
+  if (K == 0) K = keep_every_state(c, T, state) ? T : (long long)std::ceil(std::sqrt((double)T));
+  if (K > T) K = T;
+  const long long nseg = (T + K - 1) / K;
   const size_t raw_pop = pop_alloc_bytes(c);
   const size_t raw_lnk = link_bytes(c);
   const long long nl1 = std::max<long long>(1, c->n_links);
@@ -1030,9 +1046,12 @@ int adjoint_forward_impl(lbm_ctx *c, int n_steps, int checkpoint_every, const ui
     }                                                                                       \
   } while (0)
   const long long pblocks = adjoint_partial_blocks(c->N);
-  ADJ_CUDA(adj_ws_get(c, kCk, ck_bytes * nseg, (void **)&ck));
+  // one segment: every state is kept as the run goes, nothing is recomputed; only the
+  // recomputation of 16-bit storage runs on the populations themselves
+  const bool one = nseg == 1, restore = !natural && !one;
+  ADJ_CUDA(adj_ws_get(c, kCk, one ? 0 : ck_bytes * nseg, (void **)&ck));
   ADJ_CUDA(adj_ws_get(c, kSeg, state * K, (void **)&seg));
-  ADJ_CUDA(adj_ws_get(c, kFin, raw_pop + raw_lnk, (void **)&fin));
+  ADJ_CUDA(adj_ws_get(c, kFin, restore ? raw_pop + raw_lnk : 0, (void **)&fin));
   ADJ_CUDA(adj_ws_get(c, kLam0, state, (void **)&lam0));
   ADJ_CUDA(adj_ws_get(c, kLam1, state, (void **)&lam1));
   ADJ_CUDA(adj_ws_get(c, kMask, c->N, (void **)&dmask));
@@ -1076,21 +1095,19 @@ int adjoint_forward_impl(lbm_ctx *c, int n_steps, int checkpoint_every, const ui
   // last segment keeps its states as it goes, so the backward pass need not
   // recompute it.
   for (long long sgm = 0; sgm < nseg; ++sgm) {
-    if (natural)
+    if (natural && !one)
       ADJ_CUDA(launch_export_state(c->lattice, c->precision, aux_args(c), (c->t & 1) != 0,
                                    ck + ck_bytes * sgm, st));
-    else
+    else if (!one)
       ADJ_CUDA(save_raw(ck + ck_bytes * sgm));
     tp.tck[sgm] = c->t;
     const int len = (int)std::min(K, T - sgm * K);
     const int rc = sgm == nseg - 1 ? step_saving(len) : lbm_step(c, len);
     if (rc != LBM_OK) { adj_ws_free(c); return rc; }
   }
-  ADJ_CUDA(save_raw(fin));
-  // the loss (its kernel also writes lambda(T), which the backward pass recomputes)
-  ADJ_CUDA(cudaMemsetAsync(lam1, 0, state, st));
-  ADJ_CUDA(launch_export_state(c->lattice, c->precision, aux_args(c), (c->t & 1) != 0, lam1, st));
-  ADJ_CUDA(launch_loss(c->lattice, c->precision, aux_args(c), lam1, dmask, dut, lam0, dJ, st));
+  if (restore) ADJ_CUDA(save_raw(fin));
+  // the loss (the backward pass takes lambda(T) from the same kernel)
+  ADJ_CUDA(launch_loss(c->lattice, c->precision, aux_args(c), (c->t & 1) != 0, dmask, dut, nullptr, dJ, st));
   double hJ = 0.0;
   ADJ_CUDA(cudaMemcpyAsync(&hJ, dJ, sizeof(double), cudaMemcpyDeviceToHost, st));
   ADJ_CUDA(cudaStreamSynchronize(st));
@@ -1131,14 +1148,11 @@ int adjoint_backward_impl(lbm_ctx *c, double *grad_s, double *grad_q, double *gr
   const uint8_t *dmask = static_cast<const uint8_t *>(c->adj_ws[kMask].first);
   const double *dut = static_cast<const double *>(c->adj_ws[kUt].first);
   double *dJ = static_cast<double *>(c->adj_ws[kJ].first);
-  // lambda(T) from the forward end state (the current state): the state goes
-  // through lam1, which the first adjoint step overwrites; solid entries of both
+  // lambda(T) from the forward end state (the current state); solid entries of both
   // adjoint arrays stay zero
-  ADJ_CUDA(cudaMemsetAsync(lam0, 0, state, st));
   ADJ_CUDA(cudaMemsetAsync(lam1, 0, state, st));
   ADJ_CUDA(cudaMemsetAsync(dJ, 0, sizeof(double), st));
-  ADJ_CUDA(launch_export_state(c->lattice, c->precision, aux_args(c), (c->t & 1) != 0, lam1, st));
-  ADJ_CUDA(launch_loss(c->lattice, c->precision, aux_args(c), lam1, dmask, dut, lam0, dJ, st));
+  ADJ_CUDA(launch_loss(c->lattice, c->precision, aux_args(c), (c->t & 1) != 0, dmask, dut, lam0, dJ, st));
   ADJ_CUDA(cudaMemsetAsync(gpart, 0, sizeof(double) * c->Q * pblocks, st));
   ADJ_CUDA(cudaMemsetAsync(dgs, 0, sizeof(double) * 19, st));
   ADJ_CUDA(cudaMemsetAsync(dtot, 0, sizeof(double) * 2 * nl1, st));
@@ -1181,7 +1195,7 @@ int adjoint_backward_impl(lbm_ctx *c, double *grad_s, double *grad_q, double *gr
   // then step back through it
   char *lin = lam0, *lout = lam1;
   const bool last_saved = tp.last_saved;
-  tp.last_saved = false;          // the recomputation below reuses the segment buffer
+  tp.last_saved = last_saved && nseg == 1;   // a recomputation below reuses the segment buffer
   for (long long sgm = nseg - 1; sgm >= 0; --sgm) {
     const int len = (int)std::min(K, T - sgm * K);
     const bool saved = sgm == nseg - 1 && last_saved;
@@ -1213,7 +1227,7 @@ int adjoint_backward_impl(lbm_ctx *c, double *grad_s, double *grad_q, double *gr
   }
   ADJ_CUDA(launch_adjoint_finish(c->lattice, gpart, pblocks, dgs, st));
   // back to the state after the forward run
-  ADJ_CUDA(load_raw(fin));
+  if (!natural && nseg > 1) ADJ_CUDA(load_raw(fin));
   c->t = tp.t0 + T;
   std::vector<double> hgs(19), htot(2 * nl);
   ADJ_CUDA(cudaMemcpyAsync(hgs.data(), dgs, sizeof(double) * 19, cudaMemcpyDeviceToHost, st));

@@ -112,7 +112,7 @@ struct FixedCoef {
   int hi, lo;
 };
 struct FixedArgs {
-  FixedCoef row[19];         // fx_row_scale s_k / |M_k|^2 of the relaxed rows
+  FixedCoef row[19];         // fx_neq_scale 2^fx_fine s_k / |M_k|^2 of the relaxed rows
   FixedCoef inv_rho0;        // mantissa of 1/rho0 in (1/2, 1] over 4
   int quad_shift;            // right shift of j_a j_b products, plus the block exponent
   int max_exp;               // largest biased exponent of a block (below 0: none)
@@ -194,9 +194,8 @@ cudaError_t launch_export_state(int lattice, int precision, const AuxArgs &a, bo
                                 cudaStream_t st);
 cudaError_t launch_import_state(int lattice, int precision, const AuxArgs &a, const void *in,
                                 cudaStream_t st);
-cudaError_t launch_loss(int lattice, int precision, const AuxArgs &a, const void *g,
-                        const uint8_t *mask, const double *u_target, void *lam, double *J,
-                        cudaStream_t st);
+cudaError_t launch_loss(int lattice, int precision, const AuxArgs &a, bool odd, const uint8_t *mask,
+                        const double *u_target, void *lam, double *J, cudaStream_t st);
 // a cut link that takes the two-node scheme (Eq. 2.11): boundary node x_f, its
 // fluid neighbour x_l = x_f + e_i behind it, link index k, wall direction d
 struct TwoNodeLink {
