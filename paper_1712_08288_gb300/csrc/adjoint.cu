@@ -138,6 +138,7 @@ __global__ void loss_kernel(AuxArgs a, bool odd, const uint8_t *mask, const doub
 struct AdjGeo {
   const void *dcoef;          // LinkCoef<C> per link: (A', B', C', 0)
   void *acc;                  // 2 C per link: sum lambda_i, sum lambda_i (A' g_d + B' g'_i + C' g'_d)
+  FixedAdj fx;                // FP64 storage: constants of the fixed-point collision transpose
 };
 
 // position of row k among the non-conserved rows
@@ -213,6 +214,169 @@ __device__ __forceinline__ void meq_adjoint(D3Q15, const C (&smu)[15], C jx, C j
   out[3] = (a + pyz - w) * jz - c73 * smu[8] + (smu[12] * jy + smu[13] * jx) * ir0;
 }
 
+// ---------------------------------------------------------------------------
+// The collision transpose of FP64 storage in block fixed point (fixed.cuh): the state's
+// moments and the adjoint's are sums of integers, and every factor (s_k, 1/|M_k|^2,
+// the velocity) is a fixed-point product.  In FP64 this is some 400 instructions a node
+// at one warp instruction in 64 cycles per quarter SM; here the Q results, the dJ/ds
+// products and the boundary terms are FP64.  Forward and backward pass over 40 steps:
+// D3Q19 96^3 33.1 -> 16.0 ms, 56^3 7.2 -> 3.5; D2Q9 96^2 x 100 2.45 -> 2.05.
+//
+// The adjoint populations are multiples of 2^(E_l - 53), E_l their largest exponent; sums
+// with M (up to 192 times the largest) fit 62 bits.  Scaled moments and results are
+// multiples of 2^(E_l - 57).  For every s in [0, 2] and |u_a| < 0.63 (deviations under rho0/16,
+// fx_block's range) results stay below 13 times the largest adjoint value and the sums in
+// fx_meq_adjoint below 8 times (row sums of the transposed operator): 62 bits.  Nodes
+// outside these ranges take the FP64 form.
+// ---------------------------------------------------------------------------
+constexpr int kAdjIn = 53, kAdjOut = 57;
+template <class L>
+constexpr int row_abs_sum(int k) {
+  int s = 0;
+  for (int i = 0; i < L::Q; ++i) s += L::M(k, i) < 0 ? -L::M(k, i) : L::M(k, i);
+  return s;
+}
+// left shift of moment k before its products: its sum stays below 2^62
+template <class L>
+constexpr int adj_shift(int k) {
+  int sh = 0;
+  while (row_abs_sum<L>(k) << (sh + 1) <= 256) ++sh;
+  return sh;
+}
+// all rows' shifts, 3 bits each: a literal in device code
+template <class L>
+constexpr u64 adj_shifts() {
+  u64 t = 0;
+  for (int k = 0; k < L::Q; ++k) t |= (u64)adj_shift<L>(k) << (3 * k);
+  return t;
+}
+template <class L>
+struct AdjShift {
+  static constexpr u64 kAll = adj_shifts<L>();
+  static __device__ __forceinline__ constexpr int of(int k) { return (int)(kAll >> (3 * k)) & 7; }
+};
+
+}  // namespace
+
+// constants of the products: 1 / |M_k|^2 and s_k / |M_k|^2 in the units above
+template <class L>
+static FixedAdj fx_adj_args(const double *sn) {
+  FixedAdj f{};
+  for (int k = 0; k < L::Q; ++k) {
+    const int e = kAdjOut - kAdjIn - adj_shift<L>(k) + fx_fine<L>(k);
+    f.inv_n[k] = fx_coef(ldexp(1.0 / row_norm2<L>(k), e));
+    f.s_n[k] = L::conserved(k) ? FixedCoef{0, 0} : fx_coef(ldexp(sn[k], e));
+  }
+  return f;
+}
+
+namespace {
+
+// sum_k smu_k d meq_k / d(rho, j_a) as in meq_adjoint, with u_a 2^63 for j_a / rho0 and smu in its units
+// (D3Q19: rows 1, 2 times 8 and 4)
+__device__ __forceinline__ i64 adj_times(i64 v, FxHalves u) { return fx_mul(fx_halves(v << 1), u); }
+__device__ __forceinline__ FixedCoef const_sixth() { return {0x2aaaaaab, (int)0xaaaaaaab}; }       // 1/6
+__device__ __forceinline__ FixedCoef const_7_48() { return {0x25555555, 0x55555555}; }              // 7/48
+__device__ __forceinline__ void fx_meq_adjoint(D2Q9, const i64 (&smu)[9], FxHalves ux, FxHalves uy, FxHalves,
+                                               i64 (&out)[4]) {
+  out[0] = smu[2] - 2 * smu[1];
+  const i64 a = 6 * (smu[1] - smu[2]);
+  out[1] = adj_times(a + 2 * smu[7], ux) + adj_times(smu[8], uy) - smu[4];
+  out[2] = adj_times(a - 2 * smu[7], uy) + adj_times(smu[8], ux) - smu[6];
+  out[3] = 0;
+}
+__device__ __forceinline__ void fx_meq_adjoint(D3Q15, const i64 (&smu)[15], FxHalves ux, FxHalves uy, FxHalves uz,
+                                               i64 (&out)[4]) {
+  out[0] = smu[2] - smu[1];
+  const i64 a = 2 * smu[1] - 10 * smu[2], yz = a - 2 * smu[9];
+  out[1] = adj_times(a + 4 * smu[9], ux) + adj_times(smu[11], uy) + adj_times(smu[13], uz);
+  out[2] = adj_times(yz + 2 * smu[10], uy) + adj_times(smu[11], ux) + adj_times(smu[12], uz);
+  out[3] = adj_times(yz - 2 * smu[10], uz) + adj_times(smu[12], uy) + adj_times(smu[13], ux);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) out[1 + c] -= fx_mul(smu[4 + 2 * c] << 4, const_7_48());   // 7/3 smu
+}
+__device__ __forceinline__ void fx_meq_adjoint(D3Q19, const i64 (&smu)[19], FxHalves ux, FxHalves uy, FxHalves uz,
+                                               i64 (&out)[4]) {
+  out[0] = (6 * smu[2] - 11 * smu[1] + 4) >> 3;              // -11/8, 3/4
+  const i64 a = (38 * smu[1] - 22 * smu[2] + 4) >> 3;        // 38/8, -11/4
+  const i64 yz = a - 2 * smu[9] + smu[10], w = 2 * smu[11] - smu[12];
+  out[1] = adj_times(a + 4 * smu[9] - 2 * smu[10], ux) + adj_times(smu[13], uy) + adj_times(smu[15], uz);
+  out[2] = adj_times(yz + w, uy) + adj_times(smu[13], ux) + adj_times(smu[14], uz);
+  out[3] = adj_times(yz - w, uz) + adj_times(smu[14], uy) + adj_times(smu[15], ux);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) out[1 + c] -= fx_mul(smu[4 + 2 * c] << 2, const_sixth());   // 2/3 smu
+}
+
+// M^T nu with rho; rows 1 and 2 of D3Q19 arrive 8 and 4 times larger
+template <class L>
+__device__ __forceinline__ void fx_adj_back(L, const i64 (&nu)[L::Q], i64 (&t)[L::Q]) {
+  fmt<true, i64>(L{}, nu, t);
+}
+__device__ __forceinline__ void fx_adj_back(D3Q19, const i64 (&nu)[19], i64 (&t)[19]) {
+  i64 m[19];
+#pragma unroll
+  for (int k = 0; k < 19; ++k) m[k] = nu[k];
+  m[1] = m[2] = 0;
+  m[0] = 0;
+  fmt<true, i64>(D3Q19{}, m, t);
+  t[0] += nu[0] - ((30 * nu[1] + 4) >> 3) + 3 * nu[2];
+  const i64 face = nu[0] - ((11 * nu[1] + 4) >> 3) - nu[2], edge = nu[0] + nu[1] + ((nu[2] + 2) >> 2);
+#pragma unroll
+  for (int i = 1; i < 19; ++i) t[i] += i < 7 ? face : edge;
+}
+
+// Collision transpose of one node: t = M^T nu from g and lambda' (lp), and gsum_k =
+// mu_k / |M_k|^2 (m^eq_k - m_k) over -fx_neq_scale 2^-fx_fine (products in FP64: m_k - m^eq_k is
+// often small, and a product in the moments' units would lose its digits); false if
+// the node is outside the integer ranges.
+template <class L>
+__device__ __forceinline__ bool fx_adjoint(const double (&g)[L::Q], const double (&lp)[L::Q], const FixedArgs &fx,
+                                           const FixedAdj &fa, double (&t)[L::Q], double (&gsum)[L::Q]) {
+  int Eg, mx = 0;
+  if (!fx_block<L>(g, fx, Eg)) return false;
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) mx = max(mx, __double2hiint(lp[i]) & 0x7fffffff);
+  int El = mx >> 20;
+  if (mx != 0 && (El < kFxMinExp || El > 1900)) return false;
+  El = max(El, kFxMinExp);
+  i64 v[L::Q], n[L::Q];
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) v[i] = fx_from<kFxTop<L>>(g[i], Eg);
+  const auto j = fx_neq(L{}, v, n, Eg, fx);
+  const int q = fx.quad_shift - Eg - 1;
+  const FxHalves ux = fx_halves(fx_sar(fx_mul(j.x << 2, fx.inv_rho0) << 2, q));
+  const FxHalves uy = fx_halves(fx_sar(fx_mul(j.y << 2, fx.inv_rho0) << 2, q));
+  const FxHalves uz = fx_halves(fx_sar(fx_mul(j.z << 2, fx.inv_rho0) << 2, q));
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) v[i] = fx_from<kAdjIn>(lp[i], El);
+  i64 nu[L::Q], smu[L::Q];
+  {
+    i64 mu[L::Q];
+    fmoments<i64>(L{}, v, mu);
+#pragma unroll
+    for (int k = 0; k < L::Q; ++k) {
+      const i64 m = mu[k] << AdjShift<L>::of(k);
+      nu[k] = fx_mul(m, fa.inv_n[k]);
+      smu[k] = 0;
+      if (!Rows<L>::cons(k)) {
+        smu[k] = fx_mul(m, fa.s_n[k]);
+        gsum[k] = fx_to<kAdjOut>(nu[k], El) * fx_to<kFxTop<L>>(n[k], Eg);
+        nu[k] -= smu[k];
+      }
+    }
+  }
+  i64 dq[4], r[L::Q];
+  fx_meq_adjoint(L{}, smu, ux, uy, uz, dq);
+  nu[0] += dq[0];
+  nu[3] += dq[1];
+  nu[5] += dq[2];
+  if (L::D == 3) nu[7] += dq[3];
+  fx_adj_back(L{}, nu, r);
+#pragma unroll
+  for (int i = 0; i < L::Q; ++i) t[i] = fx_to<kAdjOut>(r[i], El);
+  return true;
+}
+
 // One step back in time, one node per thread.  SMALL: node indices fit in 31 bits,
 // so neighbour indices come from the node's wrapped coordinates in 32-bit
 // arithmetic.
@@ -286,8 +450,10 @@ __global__ void __launch_bounds__(kAdjThreads, sizeof(C) == 4 ? LBM_ADJ_MINB_F32
           const C av = lam_in[(long long)i * N + n];
           lp[i] += c.bb * av;
           lp[dd] += c.c * av;
-          lpre[i] += sa.one_minus_b * av;
-          lpre[dd] += c.a * av;
+          if constexpr (sizeof(C) == 4) {
+            lpre[i] += sa.one_minus_b * av;
+            lpre[dd] += c.a * av;
+          }
           // deviations suffice: A' + B' + C' = 0 removes the w_i rho0 parts
           const LinkCoef<C> dc = static_cast<const LinkCoef<C> *>(ag.dcoef)[k];
           C *acc = static_cast<C *>(ag.acc) + 2 * (long long)k;
@@ -296,38 +462,66 @@ __global__ void __launch_bounds__(kAdjThreads, sizeof(C) == 4 ? LBM_ADJ_MINB_F32
         }
       }
     }
-    // collision transpose in moment space
-    // the factored transforms (fmoments, fmt): fewer operations than the pair form
-    // (FP64: the FP64 pipe bounds the step, backward 5.60 -> 4.59 s at 128^3 x 2000;
-    // FP32: 0.349 -> 0.340 s, the gradient's difference from FP64 unchanged at 3.06e-5)
-    C m[Q], mu[Q];
-    fmoments<C>(L{}, g, m);
-    fmoments<C>(L{}, lp, mu);
-    const C jx = m[3], jy = m[5], jz = L::D == 3 ? m[7] : C(0);
-    C smu[Q], nu[Q];
-#pragma unroll
-    for (int k = 0; k < Q; ++k) {
-      if (Rows<L>::cons(k)) {
-        smu[k] = C(0);
-        mu[k] *= C(1.0 / row_norm2<L>(k));
-        continue;
-      }
-      smu[k] = sa.sn[k] * mu[k];                                      // s_k (M lambda')_k / |M_k|^2
-      mu[k] *= C(1.0 / row_norm2<L>(k));
-      gsum[k] = mu[k] * (meq(L{}, k, m[0], jx, jy, jz, ir0) - m[k]);   // d m'_k/d s_k
-      nu[k] = mu[k] - smu[k];                                         // (1 - s_k) mu_k
-    }
-    C dq[4];
-    meq_adjoint(L{}, smu, jx, jy, jz, ir0, dq);
-    nu[0] = mu[0] + dq[0];
-    nu[3] = mu[3] + dq[1];
-    nu[5] = mu[5] + dq[2];
-    if (L::D == 3) nu[7] = mu[7] + dq[3];
-    // lambda(t) = M^T nu + boundary terms
+    // collision transpose in moment space, lambda(t) = M^T nu + boundary terms
     C t[Q];
-    fmt<true, C>(L{}, nu, t);
+    bool done = false;
+    if constexpr (sizeof(C) == 8) done = fx_adjoint<L>(g, lp, sa.fx, ag.fx, t, gsum);
+    if (!done) {
+      // the factored transforms (fmoments, fmt): fewer operations than the pair form
+      // (FP32: 0.349 -> 0.340 s for the backward pass at 128^3 x 2000)
+      C m[Q], mu[Q];
+      fmoments<C>(L{}, g, m);
+      fmoments<C>(L{}, lp, mu);
+      const C jx = m[3], jy = m[5], jz = L::D == 3 ? m[7] : C(0);
+      C smu[Q], nu[Q];
 #pragma unroll
-    for (int i = 0; i < Q; ++i) lam_out[(long long)i * N + n] = lpre[i] + t[i];
+      for (int k = 0; k < Q; ++k) {
+        if (Rows<L>::cons(k)) {
+          smu[k] = C(0);
+          mu[k] *= C(1.0 / row_norm2<L>(k));
+          continue;
+        }
+        smu[k] = sa.sn[k] * mu[k];                                      // s_k (M lambda')_k / |M_k|^2
+        mu[k] *= C(1.0 / row_norm2<L>(k));
+        gsum[k] = mu[k] * (meq(L{}, k, m[0], jx, jy, jz, ir0) - m[k]);   // d m'_k/d s_k
+        nu[k] = mu[k] - smu[k];                                         // (1 - s_k) mu_k
+      }
+      C dq[4];
+      meq_adjoint(L{}, smu, jx, jy, jz, ir0, dq);
+      nu[0] = mu[0] + dq[0];
+      nu[3] = mu[3] + dq[1];
+      nu[5] = mu[5] + dq[2];
+      if (L::D == 3) nu[7] = mu[7] + dq[3];
+      fmt<true, C>(L{}, nu, t);
+      if constexpr (sizeof(C) == 8) {
+#pragma unroll
+        for (int k = 0; k < Q; ++k)
+          if (!Rows<L>::cons(k)) gsum[k] *= -(1 << fx_fine<L>(k)) / fx_neq_scale<L>(k);
+      }
+    }
+    if constexpr (sizeof(C) == 8) {
+      // boundary terms of the pre-collision values (held in lpre otherwise)
+      if (cls == kBoundary) {
+        const LinkCoef<C> *coef = static_cast<const LinkCoef<C> *>(sa.geo.coef);
+        const int bi = a.bidx[n];
+        const uint32_t mask = a.bmask[bi];
+        const int off = a.boff[bi];
+#pragma unroll
+        for (int dd = 1; dd < Q; ++dd) {
+          if (mask & (1u << dd)) {
+            const C ca = coef[off + __popc(mask & ((1u << dd) - 1u))].a;
+            const C av = lam_in[(long long)L::opp(dd) * N + n];
+            t[L::opp(dd)] += sa.one_minus_b * av;
+            t[dd] += ca * av;
+          }
+        }
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < Q; ++i) t[i] = lpre[i] + t[i];
+    }
+#pragma unroll
+    for (int i = 0; i < Q; ++i) lam_out[(long long)i * N + n] = t[i];
   }
   // dJ/ds: block sums in the compute type (FP64 arithmetic is slow on this GPU),
   // added in FP64 to this block's own partial record (no atomics)
@@ -344,11 +538,16 @@ __global__ void __launch_bounds__(kAdjThreads, sizeof(C) == 4 ? LBM_ADJ_MINB_F32
   __syncthreads();
   if (threadIdx.x < Q && !Rows<L>::cons(threadIdx.x)) {
     int slot = 0;
+    C scale = C(1);
 #pragma unroll
     for (int k = 0; k < Q; ++k)
-      if (k == (int)threadIdx.x) slot = nc_slot<L>(k);
+      if (k == (int)threadIdx.x) {
+        slot = nc_slot<L>(k);
+        if constexpr (sizeof(C) == 8) scale = -fx_neq_scale<L>(k) / (1 << fx_fine<L>(k));
+      }
     C t = C(0);
     for (int w = 0; w < kAdjThreads / 32; ++w) t += sh[w][slot];
+    if constexpr (sizeof(C) == 8) t *= scale;
     gs_part[(long long)blockIdx.x * Q + threadIdx.x] += (double)t;
   }
 }
@@ -500,13 +699,14 @@ cudaError_t launch_adjoint_step(int lattice, int precision, const SweepArgs<doub
                                 const SweepArgs<float> &a32, const AuxArgs &a, const void *dcoef,
                                 void *link_acc, const void *f, const void *lam_in, void *lam_out,
                                 double *gs_part, cudaStream_t st) {
-  const AdjGeo ag{dcoef, link_acc};
+  AdjGeo ag{dcoef, link_acc, {}};
   const unsigned blocks = (unsigned)adjoint_partial_blocks(a.N);
   const bool small = a.N < (1LL << 31);
   return with_lattice(lattice, [&](auto lat) {
     using L = decltype(lat);
     auto go = [&](const auto &sa, auto sm) {
       using C = std::remove_cv_t<std::remove_reference_t<decltype(sa.inv_rho0)>>;
+      if constexpr (sizeof(C) == 8) ag.fx = fx_adj_args<L>(sa.sn);
       adjoint_step_kernel<L, C, decltype(sm)::value><<<blocks, kAdjThreads, 0, st>>>(
           sa, a, ag, static_cast<const C *>(f), static_cast<const C *>(lam_in),
           static_cast<C *>(lam_out), gs_part);

@@ -118,6 +118,11 @@ struct FixedArgs {
   int max_exp;               // largest biased exponent of a block (below 0: none)
   int force_hi;              // high word of the largest force component
 };
+// the same for the adjoint's collision transpose (adjoint.cu)
+struct FixedAdj {
+  FixedCoef inv_n[19], s_n[19];
+};
+
 template <class C>
 struct FixedPart {};
 template <>
