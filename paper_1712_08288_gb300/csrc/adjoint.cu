@@ -41,6 +41,7 @@ __device__ __forceinline__ void atomic_add_double(double *p, double v) { atomicA
 
 template <class L, class T, class C>
 __global__ void export_state_kernel(AuxArgs a, bool odd, C *out) {
+  wait_for_previous();
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < a.N;
        n += (long long)gridDim.x * blockDim.x) {
     const int cls = a.cls[n];
@@ -72,6 +73,7 @@ template <class L, class T>
 __global__ void loss_kernel(AuxArgs a, bool odd, const uint8_t *mask, const double *u_target,
                             typename Storage<T>::C *lam, double *J) {
   using C = typename Storage<T>::C;
+  wait_for_previous();
   double acc = 0.0;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < a.N;
        n += (long long)gridDim.x * blockDim.x) {
@@ -390,6 +392,7 @@ __global__ void __launch_bounds__(kAdjThreads, sizeof(C) == 4 ? LBM_ADJ_MINB_F32
   C gsum[Q];
 #pragma unroll
   for (int k = 0; k < Q; ++k) gsum[k] = C(0);
+  wait_for_previous();
   const uint8_t cls = n < N ? a.cls[n] : (uint8_t)kSolid;
   if (cls != kSolid) {
     int x, y, z;
@@ -566,6 +569,7 @@ __global__ void __launch_bounds__(kAdjThreads, sizeof(C) == 4 ? 6 : 3)
   constexpr int Q = L::Q;
   const long long N = a.N;
   const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  wait_for_previous();
   if (n >= N) return;
   C g[Q], gp[Q];
   const uint8_t cls = a.cls[n];
@@ -623,6 +627,7 @@ __global__ void __launch_bounds__(kAdjThreads, sizeof(C) == 4 ? 6 : 3)
 // add the per-link sums of one segment to the FP64 totals and clear them
 template <class C>
 __global__ void link_flush_kernel(C *acc, double *tot, long long n) {
+  wait_for_previous();
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n;
        j += (long long)gridDim.x * blockDim.x) {
     tot[j] += (double)acc[j];
@@ -635,6 +640,7 @@ __global__ void link_flush_kernel(C *acc, double *tot, long long n) {
 template <int Q>
 __global__ void __launch_bounds__(256) gs_finish_kernel(const double *part, long long n_blocks,
                                                         double *grad_s) {
+  wait_for_previous();
   const int k = blockIdx.x;
   double v = 0.0;
   for (long long b = threadIdx.x; b < n_blocks; b += blockDim.x) v += part[b * Q + k];
@@ -663,8 +669,7 @@ cudaError_t launch_export_state(int lattice, int precision, const AuxArgs &a, bo
     return with_storage(precision, [&](auto *tp) {
       using T = std::remove_pointer_t<decltype(tp)>;
       using C = typename Storage<T>::C;
-      export_state_kernel<L, T, C><<<adj_blocks(a.N), 256, 0, st>>>(a, odd, static_cast<C *>(out));
-      return cudaGetLastError();
+      return launch_early(export_state_kernel<L, T, C>, adj_blocks(a.N), 256, 0, st, a, odd, static_cast<C *>(out));
     });
   });
 }
@@ -689,8 +694,8 @@ cudaError_t launch_loss(int lattice, int precision, const AuxArgs &a, bool odd, 
     return with_storage(precision, [&](auto *tp) {
       using T = std::remove_pointer_t<decltype(tp)>;
       using C = typename Storage<T>::C;
-      loss_kernel<L, T><<<adj_blocks(a.N), 256, 0, st>>>(a, odd, mask, u_target, static_cast<C *>(lam), J);
-      return cudaGetLastError();
+      return launch_early(loss_kernel<L, T>, adj_blocks(a.N), 256, 0, st, a, odd, mask, u_target,
+                          static_cast<C *>(lam), J);
     });
   });
 }
@@ -707,18 +712,12 @@ cudaError_t launch_adjoint_step(int lattice, int precision, const SweepArgs<doub
     auto go = [&](const auto &sa, auto sm) {
       using C = std::remove_cv_t<std::remove_reference_t<decltype(sa.inv_rho0)>>;
       if constexpr (sizeof(C) == 8) ag.fx = fx_adj_args<L>(sa.sn);
-      adjoint_step_kernel<L, C, decltype(sm)::value><<<blocks, kAdjThreads, 0, st>>>(
-          sa, a, ag, static_cast<const C *>(f), static_cast<const C *>(lam_in),
-          static_cast<C *>(lam_out), gs_part);
+      return launch_early(adjoint_step_kernel<L, C, decltype(sm)::value>, blocks, kAdjThreads, 0, st, sa, a, ag,
+                          static_cast<const C *>(f), static_cast<const C *>(lam_in), static_cast<C *>(lam_out),
+                          gs_part);
     };
-    if (precision == 0) {
-      if (small) go(a64, std::true_type{});
-      else go(a64, std::false_type{});
-    } else {
-      if (small) go(a32, std::true_type{});
-      else go(a32, std::false_type{});
-    }
-    return cudaGetLastError();
+    if (precision == 0) return small ? go(a64, std::true_type{}) : go(a64, std::false_type{});
+    return small ? go(a32, std::true_type{}) : go(a32, std::false_type{});
   });
 }
 
@@ -731,17 +730,11 @@ cudaError_t launch_recompute_step(int lattice, int precision, const SweepArgs<do
     using L = decltype(lat);
     auto go = [&](const auto &sa, auto sm) {
       using C = std::remove_cv_t<std::remove_reference_t<decltype(sa.inv_rho0)>>;
-      recompute_step_kernel<L, C, decltype(sm)::value><<<blocks, kAdjThreads, 0, st>>>(
-          sa, a, static_cast<const C *>(fin), static_cast<C *>(fout));
+      return launch_early(recompute_step_kernel<L, C, decltype(sm)::value>, blocks, kAdjThreads, 0, st, sa, a,
+                          static_cast<const C *>(fin), static_cast<C *>(fout));
     };
-    if (precision == 0) {
-      if (small) go(a64, std::true_type{});
-      else go(a64, std::false_type{});
-    } else {
-      if (small) go(a32, std::true_type{});
-      else go(a32, std::false_type{});
-    }
-    return cudaGetLastError();
+    if (precision == 0) return small ? go(a64, std::true_type{}) : go(a64, std::false_type{});
+    return small ? go(a32, std::true_type{}) : go(a32, std::false_type{});
   });
 }
 
@@ -750,20 +743,18 @@ cudaError_t launch_link_flush(int precision, void *link_acc, double *tot, long l
   if (n <= 0) return cudaSuccess;
   const int blocks = (int)std::min<long long>((n + 255) / 256, 152 * 8);
   if (precision == 0)
-    link_flush_kernel<double><<<blocks, 256, 0, st>>>(static_cast<double *>(link_acc), tot, n);
-  else
-    link_flush_kernel<float><<<blocks, 256, 0, st>>>(static_cast<float *>(link_acc), tot, n);
-  return cudaGetLastError();
+    return launch_early(link_flush_kernel<double>, blocks, 256, 0, st, static_cast<double *>(link_acc), tot, n);
+  return launch_early(link_flush_kernel<float>, blocks, 256, 0, st, static_cast<float *>(link_acc), tot, n);
 }
 
 long long adjoint_partial_blocks(long long N) { return (N + kAdjThreads - 1) / kAdjThreads; }
 
 cudaError_t launch_adjoint_finish(int lattice, const double *gs_part, long long n_blocks,
                                   double *grad_s, cudaStream_t st) {
-  if (lattice == 0) gs_finish_kernel<9><<<9, 256, 0, st>>>(gs_part, n_blocks, grad_s);
-  else if (lattice == 2) gs_finish_kernel<15><<<15, 256, 0, st>>>(gs_part, n_blocks, grad_s);
-  else gs_finish_kernel<19><<<19, 256, 0, st>>>(gs_part, n_blocks, grad_s);
-  return cudaGetLastError();
+  return with_lattice(lattice, [&](auto lat) {
+    constexpr int Q = decltype(lat)::Q;
+    return launch_early(gs_finish_kernel<Q>, Q, 256, 0, st, gs_part, n_blocks, grad_s);
+  });
 }
 
 }  // namespace lbm

@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(kMomThreads) moments_kernel(AuxArgs a, bool od
   constexpr int D = L::D;
   __shared__ double sh[kMomThreads / 32][32 * D];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  wait_for_previous();
   for (long long base = (blockIdx.x * (long long)kMomThreads) + warp * 32; base < a.N;
        base += (long long)gridDim.x * kMomThreads) {
     const int n = (int)base + lane;
@@ -114,6 +115,7 @@ template <class L, class T>
 __global__ void __launch_bounds__(kNormThreads)
     norm_partials_kernel(AuxArgs a, bool odd, const double *u_ref, double *u_prev,
                          double *partials) {
+  wait_for_previous();
   double acc[kNormFields];
 #pragma unroll
   for (int k = 0; k < kNormFields; ++k) acc[k] = 0.0;
@@ -172,6 +174,7 @@ __global__ void __launch_bounds__(kNormThreads)
 __global__ void __launch_bounds__(32 * kNormFields) norm_finish_kernel(const double *partials, int n_blocks,
                                                                      double *out) {
   const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  wait_for_previous();
   double v = 0.0;
   for (int b = lane; b < n_blocks; b += 32) {
     const double w = partials[(long long)b * kNormFields + k];
@@ -242,8 +245,7 @@ cudaError_t launch_moments(int lattice, int precision, const AuxArgs &a, bool od
     using L = decltype(lat);
     return with_storage(precision, [&](auto *tp) {
       using T = std::remove_pointer_t<decltype(tp)>;
-      moments_kernel<L, T><<<aux_blocks(a.N), kMomThreads, 0, st>>>(a, odd, rho, u);
-      return cudaGetLastError();
+      return launch_early(moments_kernel<L, T>, aux_blocks(a.N), kMomThreads, 0, st, a, odd, rho, u);
     });
   });
 }
@@ -255,17 +257,14 @@ cudaError_t launch_norm_partials(int lattice, int precision, const AuxArgs &a, b
     using L = decltype(lat);
     return with_storage(precision, [&](auto *tp) {
       using T = std::remove_pointer_t<decltype(tp)>;
-      norm_partials_kernel<L, T><<<n_blocks, kNormThreads, 0, st>>>(a, odd, u_ref, u_prev,
-                                                                      partials);
-      return cudaGetLastError();
+      return launch_early(norm_partials_kernel<L, T>, n_blocks, kNormThreads, 0, st, a, odd, u_ref, u_prev, partials);
     });
   });
 }
 
 cudaError_t launch_norm_finish(const double *partials, int n_blocks, double *out,
                                cudaStream_t st) {
-  norm_finish_kernel<<<1, 32 * kNormFields, 0, st>>>(partials, n_blocks, out);
-  return cudaGetLastError();
+  return launch_early(norm_finish_kernel, 1, 32 * kNormFields, 0, st, partials, n_blocks, out);
 }
 
 }  // namespace lbm

@@ -11,6 +11,33 @@
 
 namespace lbm {
 
+// Early launches (programmatic stream serialisation).  A kernel launched with launch_early
+// may start before the kernel in front of it in the stream has ended: its blocks take
+// their places as that kernel's leave.  It calls wait_for_previous() before it reads or writes device
+// memory, which returns once that kernel has ended and its writes are visible, and lets
+// its own successor start in turn.  This hides about 2 us of launch latency, which small
+// grids otherwise pay on every step (D2Q9 64^2 FP64: 6.2 -> 4.3 us a step; D3Q19 FP32
+// pipe L = 64: 11.3 -> 9.3).  A kernel without wait_for_previous() is never launched so.
+__device__ __forceinline__ void wait_for_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+inline cudaError_t launch_early(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                                A &&...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute early = {};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // storage type -> compute type and conversions
 template <class T>
 struct Storage;

@@ -35,6 +35,7 @@ static __device__ __align__(256) double g_noalloc_partials[kNoAllocBlocks * kFie
 template <class L, class T>
 __global__ void __launch_bounds__(kNoAllocThreads)
     noalloc_partials_kernel(AuxArgs a, bool odd, const double *u_ref, double *partials) {
+  wait_for_previous();
   double acc[kFields];
 #pragma unroll
   for (int k = 0; k < kFields; ++k) acc[k] = 0.0;
@@ -88,6 +89,7 @@ __global__ void __launch_bounds__(32 * kFields) noalloc_finish_kernel(const doub
                                                                     bool have_ref, double *out) {
   __shared__ double tot[kFields];
   const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  wait_for_previous();
   double v = 0.0;
   for (int b = lane; b < n_blocks; b += 32) {
     const double w = partials[b * kFields + k];
@@ -159,13 +161,11 @@ int error_norms_noalloc(int device, int lattice, int precision, const AuxArgs &a
     using L = decltype(lat);
     return with_storage(precision, [&](auto *tp) {
       using T = std::remove_pointer_t<decltype(tp)>;
-      noalloc_partials_kernel<L, T><<<n_blocks, kNoAllocThreads, 0, st>>>(a, odd, u_ref, scratch);
-      return cudaGetLastError();
+      return launch_early(noalloc_partials_kernel<L, T>, n_blocks, kNoAllocThreads, 0, st, a, odd, u_ref, scratch);
     });
   });
   if (e == cudaSuccess) {
-    noalloc_finish_kernel<<<1, 32 * kFields, 0, st>>>(scratch, n_blocks, u_ref != nullptr, out);
-    e = cudaGetLastError();
+    e = launch_early(noalloc_finish_kernel, 1, 32 * kFields, 0, st, scratch, n_blocks, u_ref != nullptr, out);
   }
   if (e != cudaSuccess) {
     *why = cudaGetErrorString(e);

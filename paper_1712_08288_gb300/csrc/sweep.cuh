@@ -720,6 +720,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, MinBlocks<L, T, BATCH>::v
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncwarp();
+  wait_for_previous();
   for (int s = 0; s < NS; ++s) {
     const int tile = gw + s * nw;
     if (tile < n_tiles)
@@ -1022,7 +1023,7 @@ void launch_persistent(const A &a, const TileDesc *tiles, int n_tiles, size_t sm
   }
   const int need = (n_tiles + kWarpsPerBlock - 1) / kWarpsPerBlock;
   if (grid > need) grid = need;
-  if (!prepare_only) Kernel<<<grid, threads, smem, st>>>(a, tiles, n_tiles, inst, tile_inst);
+  if (!prepare_only) launch_early(Kernel, grid, threads, smem, st, a, tiles, n_tiles, inst, tile_inst);
 }
 
 // Tile width of the single-context sweep per storage type: 64 nodes, or 32-node

@@ -25,6 +25,7 @@ __global__ void two_node_pre_kernel(const SweepArgs<typename Storage<T>::C> sa, 
                                     typename Storage<T>::C *__restrict__ delta) {
   using C = typename Storage<T>::C;
   constexpr int Q = L::Q;
+  wait_for_previous();
   const long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (j >= n_tn) return;
   const TwoNodeLink e = tn[j];
@@ -45,6 +46,7 @@ __global__ void two_node_pre_kernel(const SweepArgs<typename Storage<T>::C> sa, 
 template <class L, class T>
 __global__ void two_node_post_kernel(AuxArgs a, bool next_odd, const TwoNodeLink *__restrict__ tn,
                                      long long n_tn, const typename Storage<T>::C *__restrict__ delta) {
+  wait_for_previous();
   const long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (j >= n_tn) return;
   const TwoNodeLink e = tn[j];
@@ -70,12 +72,10 @@ cudaError_t launch_two_node(int lattice, int precision, const SweepArgs<double> 
       if constexpr (sizeof(C) == 8) sa = &a64;
       else sa = &a32;
       if (!post)
-        two_node_pre_kernel<L, T><<<tn_blocks(n_tn), kTnThreads, 0, st>>>(*sa, a, odd, tn, n_tn,
-                                                                          static_cast<C *>(delta));
-      else
-        two_node_post_kernel<L, T><<<tn_blocks(n_tn), kTnThreads, 0, st>>>(
-            a, !odd, tn, n_tn, static_cast<const C *>(delta));
-      return cudaGetLastError();
+        return launch_early(two_node_pre_kernel<L, T>, tn_blocks(n_tn), kTnThreads, 0, st, *sa, a, odd, tn, n_tn,
+                            static_cast<C *>(delta));
+      return launch_early(two_node_post_kernel<L, T>, tn_blocks(n_tn), kTnThreads, 0, st, a, !odd, tn, n_tn,
+                          static_cast<const C *>(delta));
     });
   });
 }
