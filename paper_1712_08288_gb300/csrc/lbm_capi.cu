@@ -183,7 +183,8 @@ static AuxArgs aux_args(const lbm_ctx *c) {
   a.lnk = c->lnk;
   a.rho0 = c->rho0;
   int e = 0;
-  a.inv_rho0 = std::frexp(c->rho0, &e) == 0.5 ? 1.0 / c->rho0 : 0.0;
+  const bool two = std::frexp(c->rho0, &e) == 0.5 && std::abs(e) <= 100;
+  a.rho0_exp = two ? e - 1 : AuxArgs::kNoPowerOfTwo;
   for (int k = 0; k < 3; ++k) a.g[k] = c->g[k];
   return a;
 }
@@ -349,32 +350,33 @@ static void free_geometry(lbm_ctx *c) {
   cudaFree(c->lnk); c->lnk = nullptr;
 }
 
-// A tile list in the device form (TileDesc of every tile, then TileLinks), and back.
-static cudaError_t put_tiles(const std::vector<HostTile> &t, TileDesc **dev) {
-  const size_t n = t.size(), bytes = (sizeof(TileDesc) + sizeof(TileLinks)) * n;
-  cudaError_t e = cudaMalloc((void **)dev, std::max<size_t>(sizeof(TileDesc), bytes));
+// A tile list: descriptors, and links of every tile for contexts that use them (per_link).
+struct TileList {
+  std::vector<TileDesc> d;
+  std::vector<TileLinks> k;
+  void add(const TileDesc &tile, const TileLinks *links) {
+    d.push_back(tile);
+    if (links) k.push_back(*links);
+  }
+  const TileLinks *links(size_t i) const { return k.empty() ? nullptr : &k[i]; }
+};
+
+// a list in the device form (see TileLinks), and back
+static cudaError_t put_tiles(const TileList &t, TileDesc **dev) {
+  const size_t n = t.d.size(), db = sizeof(TileDesc) * n, kb = sizeof(TileLinks) * t.k.size();
+  cudaError_t e = cudaMalloc((void **)dev, std::max<size_t>(sizeof(TileDesc), db + kb));
   if (e != cudaSuccess) *dev = nullptr;
-  if (e != cudaSuccess || n == 0) return e;
-  std::vector<unsigned char> h(bytes);
-  TileDesc *d = reinterpret_cast<TileDesc *>(h.data());
-  TileLinks *k = reinterpret_cast<TileLinks *>(d + n);
-  for (size_t i = 0; i < n; ++i) {
-    d[i] = t[i];
-    k[i] = t[i];
-  }
-  return cudaMemcpy(*dev, h.data(), bytes, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && db) e = cudaMemcpy(*dev, t.d.data(), db, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && kb) e = cudaMemcpy(*dev + n, t.k.data(), kb, cudaMemcpyHostToDevice);
+  return e;
 }
-static cudaError_t get_tiles(const TileDesc *dev, size_t n, std::vector<HostTile> &t) {
-  t.resize(n);
-  if (n == 0) return cudaSuccess;
-  std::vector<unsigned char> h((sizeof(TileDesc) + sizeof(TileLinks)) * n);
-  const cudaError_t e = cudaMemcpy(h.data(), dev, h.size(), cudaMemcpyDeviceToHost);
-  const TileDesc *d = reinterpret_cast<const TileDesc *>(h.data());
-  const TileLinks *k = reinterpret_cast<const TileLinks *>(d + n);
-  for (size_t i = 0; i < n; ++i) {
-    static_cast<TileDesc &>(t[i]) = d[i];
-    static_cast<TileLinks &>(t[i]) = k[i];
-  }
+static cudaError_t get_tiles(const TileDesc *dev, size_t n, bool links, TileList &t) {
+  t.d.resize(n);
+  t.k.resize(links ? n : 0);
+  cudaError_t e = cudaSuccess;
+  if (n) e = cudaMemcpy(t.d.data(), dev, sizeof(TileDesc) * n, cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess && n && links)
+    e = cudaMemcpy(t.k.data(), dev + n, sizeof(TileLinks) * n, cudaMemcpyDeviceToHost);
   return e;
 }
 
@@ -382,26 +384,29 @@ static cudaError_t get_tiles(const TileDesc *dev, size_t n, std::vector<HostTile
 // A half keeps the tile's link-buffer base (its records' offsets are relative to it);
 // the second half's records start after the first half's.  Lanes past a half are
 // marked solid.
-static void half_tiles(const std::vector<HostTile> &in, std::vector<HostTile> &out) {
+static void half_tiles(const TileList &in, TileList &out) {
   constexpr uint64_t kLo = 0xffffffffull;
-  out.clear();
-  out.reserve(2 * in.size());
-  for (const HostTile &d : in) {
-    HostTile a = d, h = d;
+  out.d.clear();
+  out.k.clear();
+  out.d.reserve(2 * in.d.size());
+  out.k.reserve(2 * in.k.size());
+  for (size_t i = 0; i < in.d.size(); ++i) {
+    const TileDesc &d = in.d[i];
+    TileDesc a = d, h = d;
     a.solid = d.solid | ~kLo;
     a.bnd = d.bnd & kLo;
-    a.k1 = 0;
-    h.l0 = d.l0 + d.k0;
-    h.k0 = d.k1;
-    h.k1 = 0;
-    a.dense = a.k0 > kSparseLinks;
-    h.dense = h.k0 > kSparseLinks;
     h.x0 = d.x0 + 32;
     h.rb = d.rb + __builtin_popcountll(d.bnd & kLo);
     h.solid = (d.solid >> 32) | ~kLo;
     h.bnd = d.bnd >> 32;
-    if ((a.solid & kLo) != kLo) out.push_back(a);
-    if ((h.solid & kLo) != kLo) out.push_back(h);
+    TileLinks ka{}, kh{};
+    const TileLinks *k = in.links(i);
+    if (k) {
+      ka = {k->l0, k->k0, 0, k->k0 > kSparseLinks, 0};
+      kh = {k->l0 + k->k0, k->k1, 0, k->k1 > kSparseLinks, 0};
+    }
+    if ((a.solid & kLo) != kLo) out.add(a, k ? &ka : nullptr);
+    if ((h.solid & kLo) != kLo) out.add(h, k ? &kh : nullptr);
   }
 }
 
@@ -413,20 +418,21 @@ static int upload_tiles(lbm_ctx *c, const uint8_t *solid, const std::vector<uint
   if (c->ny > 65535 || c->nz > 65535)
     return fail(c, LBM_EINVAL, "grid: ny and nz must be below 65536");
   const int nxb = (c->nx + kTileW - 1) / kTileW;
-  std::vector<HostTile> t;
-  t.reserve((size_t)nxb * c->ny * c->nz);
+  const bool with_links = per_link(c->precision);
+  TileList t;
+  t.d.reserve((size_t)nxb * c->ny * c->nz);
   std::vector<uint32_t> rec32;
   std::vector<uint16_t> ldesc;
   if (bmask) rec32.reserve(bmask->size());
-  const bool per_link = c->precision == LBM_F64;    // the sweep's link-parallel boundary
-  if (per_link) ldesc.reserve((size_t)c->n_links);
+  if (with_links) ldesc.reserve((size_t)c->n_links);
   int rb = 0;
   for (int z = 0; z < c->nz; ++z)
     for (int y = 0; y < c->ny; ++y)
       for (int xb = 0; xb < nxb; ++xb) {
         const int x0 = xb * kTileW;
         const long long row = (long long)c->nx * (y + (long long)c->ny * z);
-        HostTile d{};
+        TileDesc d{};
+        TileLinks tk{};
         d.x0 = x0;
         d.yz = y | (z << 16);
         d.rb = rb;
@@ -439,27 +445,32 @@ static int upload_tiles(lbm_ctx *c, const uint8_t *solid, const std::vector<uint
           any = true;
           if (cls && (*cls)[row + x] == kBoundary) {
             const uint32_t m = (*bmask)[rb], off = (uint32_t)(*boff)[rb];
-            if (!d.bnd) d.lb = d.l0 = (int)off;
-            (k < 32 ? d.k0 : d.k1) += (unsigned short)__builtin_popcount(m);
-            for (uint32_t w = per_link ? m : 0u; w != 0; w &= w - 1)
-              ldesc.push_back((uint16_t)((k & 31) | (__builtin_ctz(w) << kLinkDirShift)));
+            if (!d.bnd) d.lb = tk.l0 = (int)off;
+            if (with_links) {
+              (k < 32 ? tk.k0 : tk.k1) += (unsigned short)__builtin_popcount(m);
+              for (uint32_t w = m; w != 0; w &= w - 1)
+                ldesc.push_back((uint16_t)((k & 31) | (__builtin_ctz(w) << kLinkDirShift)));
+            }
             d.bnd |= 1ull << k;
             rec32.push_back(m | ((off - (uint32_t)d.lb) << kRecShift));
             ++rb;
           }
         }
-        d.dense = d.k0 > kSparseLinks || d.k1 > kSparseLinks;
-        if (any) t.push_back(d);
+        tk.dense = tk.k0 > kSparseLinks || tk.k1 > kSparseLinks;
+        if (any) t.add(d, with_links ? &tk : nullptr);
       }
-  c->n_tiles = (int)t.size();
+  c->n_tiles = (int)t.d.size();
   cudaFree(c->tiles);
   c->tiles = nullptr;
-  std::vector<HostTile> th;
-  half_tiles(t, th);
-  c->n_tiles_half = (int)th.size();
   cudaFree(c->tiles_half);
   c->tiles_half = nullptr;
-  CUDA_OR_FAIL(c, put_tiles(th, &c->tiles_half));
+  c->n_tiles_half = 0;
+  if (half_tiled(c->precision)) {
+    TileList th;
+    half_tiles(t, th);
+    c->n_tiles_half = (int)th.d.size();
+    CUDA_OR_FAIL(c, put_tiles(th, &c->tiles_half));
+  }
   cudaFree(c->rec32);
   c->rec32 = nullptr;
   CUDA_OR_FAIL(c, put_tiles(t, &c->tiles));
@@ -1330,7 +1341,7 @@ struct lbm_batch {
   std::vector<lbm_ctx *> ctx;
   int lattice = 0, precision = 0, device = 0;
   cudaStream_t stream = nullptr;
-  std::vector<std::vector<HostTile>> host_tiles;   // per context
+  std::vector<TileList> host_tiles;   // per context
   std::vector<long long> versions;
   void *inst = nullptr;          // SweepArgs per context (compute type of the precision)
   BatchList lists[kBatchClasses];  // tile lists per kernel class (batch_upload)
@@ -1393,19 +1404,19 @@ static int batch_upload(lbm_batch *b) {
     }
   // the members' tiles in the batch's tile width (64-bit slot indices: 64 only)
   const bool halves = b->tile_w == 32 && !b->big;
-  std::vector<std::vector<HostTile>> halved(halves ? n : 0);
+  std::vector<TileList> halved(halves ? n : 0);
   for (int k = 0; k < (halves ? n : 0); ++k) half_tiles(b->host_tiles[k], halved[k]);
-  const std::vector<std::vector<HostTile>> &mt = halves ? halved : b->host_tiles;
+  const std::vector<TileList> &mt = halves ? halved : b->host_tiles;
   std::vector<int> ctx_order(n);
   for (int k = 0; k < n; ++k) ctx_order[k] = k;
   if (b->order == 2)
     std::stable_sort(ctx_order.begin(), ctx_order.end(), [&](int p, int q) {
-      return mt[p].size() > mt[q].size();
+      return mt[p].d.size() > mt[q].d.size();
     });
   b->n_tiles = 0;
   for (int cl = 0; cl < kBatchClasses; ++cl) {
     BatchList &bl = b->lists[cl];
-    std::vector<HostTile> t;
+    TileList t;
     std::vector<int> ti;
     if (b->order == 1) {
       // round-robin: one tile of every member of the class in turn
@@ -1414,8 +1425,9 @@ static int batch_upload(lbm_batch *b) {
       while (more) {
         more = false;
         for (int k : ctx_order)
-          if (cls_of[k] == cl && pos[k] < mt[k].size()) {
-            t.push_back(mt[k][pos[k]++]);
+          if (cls_of[k] == cl && pos[k] < mt[k].d.size()) {
+            t.add(mt[k].d[pos[k]], mt[k].links(pos[k]));
+            ++pos[k];
             ti.push_back(k);
             more = true;
           }
@@ -1423,8 +1435,8 @@ static int batch_upload(lbm_batch *b) {
     } else {
       for (int k : ctx_order)
         if (cls_of[k] == cl)
-          for (const HostTile &d : mt[k]) {
-            t.push_back(d);
+          for (size_t i = 0; i < mt[k].d.size(); ++i) {
+            t.add(mt[k].d[i], mt[k].links(i));
             ti.push_back(k);
           }
     }
@@ -1432,9 +1444,9 @@ static int batch_upload(lbm_batch *b) {
     cudaFree(bl.tile_inst);
     bl.tiles = nullptr;
     bl.tile_inst = nullptr;
-    bl.n = (int)t.size();
+    bl.n = (int)t.d.size();
     b->n_tiles += bl.n;
-    if (t.empty()) continue;
+    if (t.d.empty()) continue;
     BCUDA(b, put_tiles(t, &bl.tiles));
     BCUDA(b, cudaMalloc((void **)&bl.tile_inst, sizeof(int) * ti.size()));
     BCUDA(b, cudaMemcpy(bl.tile_inst, ti.data(), sizeof(int) * ti.size(), cudaMemcpyHostToDevice));
@@ -1464,7 +1476,7 @@ static int batch_refresh_if_needed(lbm_batch *b) {
   // geometry may have changed: fetch the tile lists again
   for (size_t k = 0; k < b->ctx.size(); ++k) {
     lbm_ctx *c = b->ctx[k];
-    BCUDA(b, get_tiles(c->tiles, c->n_tiles, b->host_tiles[k]));
+    BCUDA(b, get_tiles(c->tiles, c->n_tiles, per_link(c->precision), b->host_tiles[k]));
   }
   int rc = batch_upload(b);
   if (rc == LBM_OK) rc = batch_upload_args(b);

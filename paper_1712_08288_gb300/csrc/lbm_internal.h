@@ -47,14 +47,17 @@ struct alignas(16) TileDesc {
 };
 // A tile's links for the link-parallel boundary (FP64 storage): first link, counts of
 // the two 32-node halves (a half tile has one), and whether a half has more than
-// kSparseLinks.  A list of n tiles on the device is n TileDesc, then n TileLinks (apart,
-// since the sweeps that do not need them lose 3 % to the longer descriptors).
+// kSparseLinks.  A list of n tiles on the device is n TileDesc, then (FP64) n TileLinks:
+// sweeps that do not need them lose 3 % to longer descriptors.
 struct alignas(16) TileLinks {
   int l0;
   unsigned short k0, k1;
   int dense, pad;
 };
-struct HostTile : TileDesc, TileLinks {};
+// whether contexts of a storage precision use the link-parallel boundary, and 32-node half tiles
+// when they step alone (FP64)
+constexpr bool per_link(int precision) { return precision == 0; }
+constexpr bool half_tiled(int precision) { return precision == 0; }
 constexpr int kSparseLinks = 64;
 // descriptor of a link: node within its 32-node half in bits 0..4, direction above
 constexpr int kLinkDirShift = 5;
@@ -168,7 +171,8 @@ struct AuxArgs {
   const int32_t *boff;
   const void *lnk;
   double rho0;
-  double inv_rho0;           // 1 / rho0 where rho0 is a power of two, else 0
+  static constexpr int kNoPowerOfTwo = 1 << 20;
+  int rho0_exp;              // log2(rho0) where rho0 is a power of two in [2^-100, 2^100], else kNoPowerOfTwo
   double g[3];
 };
 

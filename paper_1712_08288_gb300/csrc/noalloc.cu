@@ -39,31 +39,32 @@ __global__ void __launch_bounds__(kNoAllocThreads)
   double acc[kFields];
 #pragma unroll
   for (int k = 0; k < kFields; ++k) acc[k] = 0.0;
+  i64 worst = 0;
   for (long long n = blockIdx.x * (long long)kNoAllocThreads + threadIdx.x; n < a.N;
        n += (long long)gridDim.x * kNoAllocThreads) {
     const int cls = a.cls[n];
     if (cls == kSolid) continue;
     typename Storage<T>::C g[L::Q];
     load_node<L, T>(g, (int)n, cls, odd, a);
-    double drho, j[3];
-    node_sums<L>(g, drho, j);
-    const double rho = a.rho0 + drho;
-    if (!isfinite(rho)) acc[7] += 1.0;
+    const NodeSums s = node_sums<L>(g, a);
+    const double rho = a.rho0 + s.drho;
+    if (!finite_bits(rho)) acc[7] += 1.0;
     acc[3] += rho;
-    acc[4] += j[0];
-    acc[5] += j[1];
-    acc[6] += j[2];
+    acc[4] += s.j[0];
+    acc[5] += s.j[1];
+    acc[6] += s.j[2];
     if (u_ref) {
 #pragma unroll
       for (int k = 0; k < L::D; ++k) {
-        const double uk = velocity(j[k], a, k);
+        const double uk = velocity(s, a, k);
         const double df = u_ref[n * L::D + k] - uk;
         acc[0] += df * df;
         acc[1] += u_ref[n * L::D + k] * u_ref[n * L::D + k];
-        acc[2] = fmax(acc[2], fabs(df));
+        worst = max(worst, magnitude_bits(df));
       }
     }
   }
+  acc[2] = __longlong_as_double(worst);
   __shared__ double sh[kNoAllocThreads / 32][kFields];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -80,6 +81,7 @@ __global__ void __launch_bounds__(kNoAllocThreads)
     const int k = threadIdx.x;
     double v = sh[0][k];
     for (int w = 1; w < kNoAllocThreads / 32; ++w) v = (k == 2) ? fmax(v, sh[w][k]) : v + sh[w][k];
+    if (k >= 4 && k <= 6) v *= momentum_factor(a);
     partials[blockIdx.x * kFields + k] = v;
   }
 }

@@ -62,24 +62,39 @@ __device__ __forceinline__ void load_node(typename Storage<T>::C (&g)[L::Q], int
   }
 }
 
-// sums of the integers, times 2^scale
+// rho - rho0 and j / rho0 of a node, and j in the form that sums add up: j / rho0 where
+// rho0 is a power of two (exact), j otherwise (momentum_factor() undoes it)
+struct NodeSums {
+  double drho, u[3], j[3];
+};
+__device__ __forceinline__ double momentum_factor(const AuxArgs &a) {
+  return a.rho0_exp != AuxArgs::kNoPowerOfTwo ? a.rho0 : 1.0;
+}
+
+// Sums of the integers times 2^scale.  A power of two rho0 divides j exactly through the
+// exponents (AuxArgs::rho0_exp), at no cost.
 template <class L>
-__device__ __forceinline__ void scaled_sums(const i64 (&v)[L::Q], int scale, double &drho, double (&j)[3]) {
+__device__ __forceinline__ NodeSums scaled_sums(const i64 (&v)[L::Q], int scale, const AuxArgs &a) {
   i64 m[L::Q];
   fmoments<i64>(L{}, v, m);   // rho and j are used, the rest is never computed
-  auto to = [&](i64 x) {
+  auto to = [&](i64 x, int sc) {
     const double d = (double)x;
-    return __hiloint2double(x != 0 ? __double2hiint(d) + (scale << 20) : 0, __double2loint(d));
+    return __hiloint2double(x != 0 ? __double2hiint(d) + (sc << 20) : 0, __double2loint(d));
   };
-  drho = to(m[0]);
-  j[0] = to(m[3]);
-  j[1] = to(m[5]);
-  j[2] = L::D == 3 ? to(m[7]) : 0.0;
+  const bool two = a.rho0_exp != AuxArgs::kNoPowerOfTwo;
+  const int su = two ? scale - a.rho0_exp : scale;
+  const double x = to(m[3], su), y = to(m[5], su), z = L::D == 3 ? to(m[7], su) : 0.0;
+  NodeSums r = {to(m[0], scale), {x, y, z}, {x, y, z}};
+  if (!two) {
+#pragma unroll
+    for (int k = 0; k < L::D; ++k) r.u[k] /= a.rho0;
+  }
+  return r;
 }
 
 template <class L, class C>
-__device__ __forceinline__ void plain_sums(const C (&g)[L::Q], double &drho, double (&j)[3]) {
-  drho = j[0] = j[1] = j[2] = 0.0;
+__device__ __forceinline__ NodeSums plain_sums(const C (&g)[L::Q], const AuxArgs &a) {
+  double drho = 0.0, j[3] = {0.0, 0.0, 0.0};
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) {
     const double v = (double)g[i];
@@ -88,18 +103,23 @@ __device__ __forceinline__ void plain_sums(const C (&g)[L::Q], double &drho, dou
     if (L::ey(i) != 0) j[1] += L::ey(i) * v;
     if (L::ez(i) != 0) j[2] += L::ez(i) * v;
   }
+  NodeSums r = {drho, {j[0] / a.rho0, j[1] / a.rho0, j[2] / a.rho0}, {j[0], j[1], j[2]}};
+  if (a.rho0_exp != AuxArgs::kNoPowerOfTwo) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) r.j[k] = r.u[k];
+  }
+  return r;
 }
 
 template <class L>
-__device__ __forceinline__ void node_sums(const float (&g)[L::Q], double &drho, double (&j)[3]) {
+__device__ __forceinline__ NodeSums node_sums(const float (&g)[L::Q], const AuxArgs &a) {
   constexpr int kTop = 57;        // 19 (2^58) < 2^63
   unsigned mx = 0;
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) mx = max(mx, __float_as_uint(g[i]) & 0x7fffffffu);
   const int E = (int)(mx >> 23);
   if (mx != 0 && (E < 64 || E == 255)) {   // below 64 a subnormal number could count
-    plain_sums<L>(g, drho, j);
-    return;
+    return plain_sums<L>(g, a);
   }
   i64 v[L::Q];
 #pragma unroll
@@ -110,31 +130,34 @@ __device__ __forceinline__ void node_sums(const float (&g)[L::Q], double &drho, 
     const i64 s = (i64)((int)b >> 31);
     v[i] = ((i64)fx_shr(top, d) ^ s) - s;
   }
-  scaled_sums<L>(v, max(E, 64) - 127 - kTop, drho, j);
+  return scaled_sums<L>(v, max(E, 64) - 127 - kTop, a);
 }
 
 template <class L>
-__device__ __forceinline__ void node_sums(const double (&g)[L::Q], double &drho, double (&j)[3]) {
+__device__ __forceinline__ NodeSums node_sums(const double (&g)[L::Q], const AuxArgs &a) {
   constexpr int kTop = 57;
   int mx = 0;
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) mx = max(mx, __double2hiint(g[i]) & 0x7fffffff);
   const int E = mx >> 20;
-  if (mx != 0 && (E < kFxMinExp || E == 2047)) {
-    plain_sums<L>(g, drho, j);
-    return;
-  }
+  if (mx != 0 && (E < kFxMinExp || E == 2047)) return plain_sums<L>(g, a);
   i64 v[L::Q];
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) v[i] = fx_from<kTop>(g[i], max(E, kFxMinExp));
-  scaled_sums<L>(v, max(E, kFxMinExp) - 1023 - kTop, drho, j);
+  return scaled_sums<L>(v, max(E, kFxMinExp) - 1023 - kTop, a);
 }
 
-// velocity component: j / rho0 + g / 2.  A power of two is divided by exactly by its
-// reciprocal (one instruction instead of a division's dozen).
-__device__ __forceinline__ double velocity(double j, const AuxArgs &a, int k) {
-  const double u = a.inv_rho0 != 0.0 ? j * a.inv_rho0 : j / a.rho0;
-  return a.g[k] != 0.0 ? u + 0.5 * a.g[k] : u;
+// reported velocity component: j / rho0 + g / 2
+__device__ __forceinline__ double velocity(const NodeSums &s, const AuxArgs &a, int k) {
+  return a.g[k] != 0.0 ? s.u[k] + 0.5 * a.g[k] : s.u[k];
 }
+
+// |x| as an ordered integer, 0 for NaN (which fmax ignores): maxima and finiteness without
+// the FP64 pipe
+__device__ __forceinline__ i64 magnitude_bits(double x) {
+  const i64 b = __double_as_longlong(x) & 0x7fffffffffffffffll;
+  return b > 0x7ff0000000000000ll ? 0 : b;
+}
+__device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 
 }  // namespace lbm

@@ -506,7 +506,7 @@ static_assert((StageShape<__half>::kWidth * sizeof(__half)) % 16 == 0, "window s
 // (FP32: pipe L = 256, 271 -> 288 us; ensemble of 32 annuli, 62 -> 69).
 template <class T>
 __host__ __device__ constexpr bool link_parallel() {
-  return sizeof(T) == 8;
+  return per_link(sizeof(T) == 8 ? 0 : 1);
 }
 static_assert(StageShape<double, 32>::kRecs * 4 >= kSparseLinks * 2 + 16 && StageShape<double>::kRecs * 4 >= 2 * kSparseLinks * 2 + 16,
               "the link descriptors of a sparse tile fit the record window");
@@ -1029,18 +1029,9 @@ void launch_persistent(const A &a, const TileDesc *tiles, int n_tiles, size_t sm
 // Tile width of the single-context sweep per storage type: 64 nodes, or 32-node
 // half tiles for FP64 storage (see StageShape; on the L = 256 pipe 3.99 instead of
 // 4.01 ms per step, the same with 64-node tiles in one stage or 32-node tiles in 3).
-#ifndef LBM_TILEW_F64
-#define LBM_TILEW_F64 32
-#endif
-#ifndef LBM_TILEW_4B
-#define LBM_TILEW_4B 64
-#endif
-#ifndef LBM_TILEW_2B
-#define LBM_TILEW_2B 64
-#endif
 template <class T>
 constexpr int single_tile_w() {
-  return sizeof(T) == 8 ? LBM_TILEW_F64 : (sizeof(T) == 4 ? LBM_TILEW_4B : LBM_TILEW_2B);
+  return half_tiled(sizeof(T) == 8 ? 0 : 1) ? 32 : kTileW;
 }
 
 template <class L, class T>
