@@ -154,29 +154,6 @@ __host__ __device__ constexpr int nc_slot(int k) {
 static_assert(nc_slot<D3Q19>(19) <= 16 && nc_slot<D3Q15>(15) <= 16 && nc_slot<D2Q9>(9) <= 16,
               "at most 16 relaxed rows");
 
-// Transposing warp reduction of 16 values per lane: at each of the offsets 16, 8,
-// 4, 2 a lane keeps the half of its values that its lane bit selects and adds the
-// partner's copy of that half; the pair (l, l^1) is combined last.  Lane l returns
-// the warp sum of v[l >> 1]: 16 shuffles instead of 16 x 5.
-template <class C>
-__device__ __forceinline__ C warp_sum16(const C (&v)[16]) {
-  const unsigned lane = threadIdx.x & 31u;
-  const bool b4 = lane & 16u, b3 = lane & 8u, b2 = lane & 4u, b1 = lane & 2u;
-  C a8[8], a4[4], a2[2];
-#pragma unroll
-  for (int j = 0; j < 8; ++j)
-    a8[j] = (b4 ? v[j + 8] : v[j]) + __shfl_xor_sync(0xffffffffu, b4 ? v[j] : v[j + 8], 16);
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-    a4[j] = (b3 ? a8[j + 4] : a8[j]) + __shfl_xor_sync(0xffffffffu, b3 ? a8[j] : a8[j + 4], 8);
-#pragma unroll
-  for (int j = 0; j < 2; ++j)
-    a2[j] = (b2 ? a4[j + 2] : a4[j]) + __shfl_xor_sync(0xffffffffu, b2 ? a4[j] : a4[j + 2], 4);
-  C r = (b1 ? a2[1] : a2[0]) + __shfl_xor_sync(0xffffffffu, b1 ? a2[0] : a2[1], 2);
-  r += __shfl_xor_sync(0xffffffffu, r, 1);
-  return r;
-}
-
 // sum_k smu_k * d meq_k / d(rho, j_x, j_y, j_z) for the equilibrium moments of
 // meq() (deviation form), smu_k = s_k mu_k on the non-conserved rows
 template <class C>

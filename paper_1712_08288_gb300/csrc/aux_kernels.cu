@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kMomThreads) moments_kernel(AuxArgs a, bool od
 constexpr int kNormThreads = 256;
 
 template <class L, class T>
-__global__ void __launch_bounds__(kNormThreads)
+__global__ void __launch_bounds__(kNormThreads, 3)
     norm_partials_kernel(AuxArgs a, bool odd, const double *u_ref, double *u_prev,
                          double *partials) {
   wait_for_previous();
@@ -153,19 +153,16 @@ __global__ void __launch_bounds__(kNormThreads)
       u_prev[n * L::D + k] = uk;
     }
   }
-  acc[2] = __longlong_as_double(worst);
-  // block reduction (fixed order -> deterministic)
+  // block reduction (fixed order -> deterministic); 16 additions a lane for the 9 sums
   __shared__ double sh[kNormThreads / 32][kNormFields];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double v16[16];
 #pragma unroll
-  for (int k = 0; k < kNormFields; ++k) {
-    double v = acc[k];
-    for (int o = 16; o > 0; o >>= 1) {
-      const double w = __shfl_down_sync(0xffffffffu, v, o);
-      v = (k == 2) ? fmax(v, w) : v + w;
-    }
-    if (lane == 0) sh[warp][k] = v;
-  }
+  for (int k = 0; k < 16; ++k) v16[k] = k < kNormFields ? acc[k] : 0.0;
+  const double sum = warp_sum16(v16);
+  worst = warp_max(worst);
+  const int field = lane >> 1;
+  if ((lane & 1) == 0 && field < kNormFields) sh[warp][field] = field == 2 ? __longlong_as_double(worst) : sum;
   __syncthreads();
   if (threadIdx.x < kNormFields) {
     const int k = threadIdx.x;
@@ -182,6 +179,7 @@ __global__ void __launch_bounds__(32 * kNormFields) norm_finish_kernel(const dou
   const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
   wait_for_previous();
   double v = 0.0;
+#pragma unroll 8
   for (int b = lane; b < n_blocks; b += 32) {
     const double w = partials[(long long)b * kNormFields + k];
     v = (k == 2) ? fmax(v, w) : v + w;
@@ -204,7 +202,7 @@ int aux_blocks(long long N) {
 
 int norm_blocks_for(long long N) {
   long long b = (N + kNormThreads - 1) / kNormThreads;
-  if (b > 152 * 8) b = 152 * 8;
+  if (b > 152 * 6) b = 152 * 6;   // whole waves of 3 blocks per SM
   if (b < 1) b = 1;
   return (int)b;
 }

@@ -114,6 +114,46 @@ __device__ __forceinline__ const T *population_address(int i, long long n, bool 
          wrap_index(x, y, z, -L::ex(i), -L::ey(i), -L::ez(i), a.nx, a.ny, a.nz, a.sy, a.sz);
 }
 
+// Transposing warp reduction of 16 values per lane: at each of the offsets 16, 8,
+// 4, 2 a lane keeps the half of its values that its lane bit selects and adds the
+// partner's copy of that half; the pair (l, l^1) is combined last.  Lane l returns
+// the warp sum of v[l >> 1]: 16 shuffles instead of 16 x 5.
+template <class C>
+__device__ __forceinline__ C warp_sum16(const C (&v)[16]) {
+  const unsigned lane = threadIdx.x & 31u;
+  const bool b4 = lane & 16u, b3 = lane & 8u, b2 = lane & 4u, b1 = lane & 2u;
+  C a8[8], a4[4], a2[2];
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    a8[j] = (b4 ? v[j + 8] : v[j]) + __shfl_xor_sync(0xffffffffu, b4 ? v[j] : v[j + 8], 16);
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    a4[j] = (b3 ? a8[j + 4] : a8[j]) + __shfl_xor_sync(0xffffffffu, b3 ? a8[j] : a8[j + 4], 8);
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+    a2[j] = (b2 ? a4[j + 2] : a4[j]) + __shfl_xor_sync(0xffffffffu, b2 ? a4[j] : a4[j + 2], 4);
+  C r = (b1 ? a2[1] : a2[0]) + __shfl_xor_sync(0xffffffffu, b1 ? a2[0] : a2[1], 2);
+  r += __shfl_xor_sync(0xffffffffu, r, 1);
+  return r;
+}
+// The same for 8 values: lane l returns the warp sum of v[l >> 2].
+template <class C>
+__device__ __forceinline__ C warp_sum8(const C (&v)[8]) {
+  const unsigned lane = threadIdx.x & 31u;
+  const bool b4 = lane & 16u, b3 = lane & 8u, b2 = lane & 4u;
+  C a4[4], a2[2];
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    a4[j] = (b4 ? v[j + 4] : v[j]) + __shfl_xor_sync(0xffffffffu, b4 ? v[j] : v[j + 4], 16);
+#pragma unroll
+  for (int j = 0; j < 2; ++j)
+    a2[j] = (b3 ? a4[j + 2] : a4[j]) + __shfl_xor_sync(0xffffffffu, b3 ? a4[j] : a4[j + 2], 8);
+  C r = (b2 ? a2[1] : a2[0]) + __shfl_xor_sync(0xffffffffu, b2 ? a2[0] : a2[1], 4);
+  r += __shfl_xor_sync(0xffffffffu, r, 2);
+  r += __shfl_xor_sync(0xffffffffu, r, 1);
+  return r;
+}
+
 // dispatch helper: storage type for an lbm_precision value
 template <class F>
 __host__ inline cudaError_t with_storage(int precision, F &&f) {

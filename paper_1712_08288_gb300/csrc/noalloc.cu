@@ -33,7 +33,7 @@ constexpr int kFields = 8;  // sum|u_ref-u|^2, sum|u_ref|^2, max|u_ref-u|, sum r
 static __device__ __align__(256) double g_noalloc_partials[kNoAllocBlocks * kFields];
 
 template <class L, class T>
-__global__ void __launch_bounds__(kNoAllocThreads)
+__global__ void __launch_bounds__(kNoAllocThreads, 3)
     noalloc_partials_kernel(AuxArgs a, bool odd, const double *u_ref, double *partials) {
   wait_for_previous();
   double acc[kFields];
@@ -64,18 +64,13 @@ __global__ void __launch_bounds__(kNoAllocThreads)
       }
     }
   }
-  acc[2] = __longlong_as_double(worst);
+  // 9 additions a lane for the 7 sums (a shuffle tree per field would take 35)
   __shared__ double sh[kNoAllocThreads / 32][kFields];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < kFields; ++k) {
-    double v = acc[k];
-    for (int o = 16; o > 0; o >>= 1) {
-      const double w = __shfl_down_sync(0xffffffffu, v, o);
-      v = (k == 2) ? fmax(v, w) : v + w;
-    }
-    if (lane == 0) sh[warp][k] = v;
-  }
+  static_assert(kFields == 8, "fields of a record");
+  const double sum = warp_sum8(acc);
+  worst = warp_max(worst);
+  if ((lane & 3) == 0) sh[warp][lane >> 2] = (lane >> 2) == 2 ? __longlong_as_double(worst) : sum;
   __syncthreads();
   if (threadIdx.x < kFields) {
     const int k = threadIdx.x;
@@ -93,6 +88,7 @@ __global__ void __launch_bounds__(32 * kFields) noalloc_finish_kernel(const doub
   const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
   wait_for_previous();
   double v = 0.0;
+#pragma unroll 8
   for (int b = lane; b < n_blocks; b += 32) {
     const double w = partials[b * kFields + k];
     v = (k == 2) ? fmax(v, w) : v + w;
@@ -103,15 +99,19 @@ __global__ void __launch_bounds__(32 * kFields) noalloc_finish_kernel(const doub
   }
   if (lane == 0) tot[k] = v;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    const double nan = __longlong_as_double(0x7ff8000000000000LL);
-    out[0] = have_ref ? sqrt(tot[0]) / sqrt(tot[1]) : nan;
-    out[1] = have_ref ? tot[2] : nan;
-    out[2] = tot[3];
-    out[3] = tot[4];
-    out[4] = tot[5];
-    out[5] = tot[6];
-    out[6] = tot[7];
+  if (threadIdx.x < 32) {
+    // the two square roots side by side
+    const double root = sqrt(tot[lane & 1]), den = __shfl_sync(0xffffffffu, root, 1);
+    if (lane == 0) {
+      const double nan = __longlong_as_double(0x7ff8000000000000LL);
+      out[0] = have_ref ? root / den : nan;
+      out[1] = have_ref ? tot[2] : nan;
+      out[2] = tot[3];
+      out[3] = tot[4];
+      out[4] = tot[5];
+      out[5] = tot[6];
+      out[6] = tot[7];
+    }
   }
 }
 
@@ -156,9 +156,11 @@ int error_norms_noalloc(int device, int lattice, int precision, const AuxArgs &a
     *why = cudaGetErrorString(e);
     return LBM_ECUDA;
   }
-  // one record per block; as many blocks as the array has records, fewer on small grids
+  // one record per block: whole waves of 3 blocks per SM, fewer blocks on small grids
+  constexpr int kBlocks = 152 * 6;
+  static_assert(kBlocks <= kNoAllocBlocks, "the array holds a record per block");
   const long long want = (a.N + kNoAllocThreads - 1) / kNoAllocThreads;
-  const int n_blocks = (int)(want < kNoAllocBlocks ? want : kNoAllocBlocks);
+  const int n_blocks = (int)(want < kBlocks ? want : kBlocks);
   e = with_lattice(lattice, [&](auto lat) {
     using L = decltype(lat);
     return with_storage(precision, [&](auto *tp) {

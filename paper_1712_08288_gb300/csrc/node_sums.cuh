@@ -158,6 +158,10 @@ __device__ __forceinline__ i64 magnitude_bits(double x) {
   const i64 b = __double_as_longlong(x) & 0x7fffffffffffffffll;
   return b > 0x7ff0000000000000ll ? 0 : b;
 }
+__device__ __forceinline__ i64 warp_max(i64 v) {
+  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
 __device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 
 }  // namespace lbm
