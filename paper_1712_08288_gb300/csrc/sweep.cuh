@@ -715,16 +715,30 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, MinBlocks<L, T, BATCH>::v
   const TileLinks *const links = reinterpret_cast<const TileLinks *>(tiles + n_tiles);
   const int gw = blockIdx.x * kWarpsPerBlock + warp;
   const int nw = gridDim.x * kWarpsPerBlock;
+  // The first tiles' descriptors come in before the wait for the kernel in front: they
+  // change only by host copies, which this launch is ordered behind.
+  TileDesc first[NS];
+  TileLinks first_links[NS];
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    first[s] = TileDesc{};
+    first_links[s] = TileLinks{};
+    if (gw + s * nw < n_tiles) {
+      first[s] = tiles[gw + s * nw];
+      if constexpr (link_parallel<T>()) first_links[s] = links[gw + s * nw];
+    }
+  }
   if (lane == 0) {
     for (int s = 0; s < NS; ++s) mbar_init(&bars[s], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncwarp();
   wait_for_previous();
+#pragma unroll
   for (int s = 0; s < NS; ++s) {
     const int tile = gw + s * nw;
     if (tile < n_tiles)
-      issue_tile<L, T, ODD, ALIGNED, I, TW>(args_for<BATCH>(a, inst, tile_inst, tile), tiles[tile], links + tile,
+      issue_tile<L, T, ODD, ALIGNED, I, TW>(args_for<BATCH>(a, inst, tile_inst, tile), first[s], first_links + s,
                                wsm + s * SL::kStage, offs + s * NO, &bars[s]);
   }
 
