@@ -40,7 +40,7 @@ template <class L>
 constexpr int kFxTop = L::Q == 9 ? 57 : 56;
 constexpr int kFxMinExp = 128;  // smallest biased exponent of a block
 
-// logical right shift whose amount may exceed 63 (result 0)
+// right shifts whose amount may exceed 63 (result 0, or -1 for negative x); the hardware clamps
 LBM_HD u64 fx_shr(u64 x, int n) {
 #ifdef __CUDA_ARCH__
   u64 r;
@@ -97,8 +97,8 @@ template <int kTop>
 LBM_HD double fx_to(i64 v, int E) {
   const double x = (double)v;
 #ifdef __CUDA_ARCH__
-  const int hi = __double2hiint(x);
-  return __hiloint2double(v != 0 ? hi + ((E - 1023 - kTop) << 20) : 0, __double2loint(x));
+  const int hi = __double2hiint(x);       // 0 only for x = 0
+  return __hiloint2double(hi != 0 ? hi + ((E - 1023 - kTop) << 20) : 0, __double2loint(x));
 #else
   return v != 0 ? ldexp(x, E - 1023 - kTop) : 0.0;
 #endif

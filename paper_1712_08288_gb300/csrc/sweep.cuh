@@ -441,16 +441,17 @@ __device__ __forceinline__ void bulk_copy_g2s(void *dst, const void *src, uint32
 // TW + 16/sizeof(T) elements, start aligned down to 16 bytes), filled by bulk copies
 // that complete on the warp's own mbarrier.  32-node tiles take more stages with 4-
 // and 2-byte storage (3 and 5): a warp keeps most of its bytes in flight while a
-// block still fits the shared memory of the 64-node layout.  FP64 storage keeps 2
-// stages in 32-node tiles: its sweep is bound by the FP64 pipe, and half the shared
-// memory doubles the blocks per SM (4 instead of 2).  Warps never wait for each other.
+// block still fits the shared memory of the 64-node layout.  FP64 storage takes 2
+// stages of 32-node tiles or one of 64-node tiles, so that 4 blocks fit an SM (2 stages of
+// 64-node tiles at 2 blocks: D2Q9 2048^2 95 against 85 us a step).  Warps never wait
+// for each other.
 constexpr int kWarpsPerBlock = 4;
 
 #ifndef LBM_STAGES_4B
 #define LBM_STAGES_4B 2
 #endif
 #ifndef LBM_STAGES_8B
-#define LBM_STAGES_8B 2
+#define LBM_STAGES_8B 1
 #endif
 #ifndef LBM_STAGES_8B_32
 #define LBM_STAGES_8B_32 2
@@ -662,13 +663,12 @@ struct MinBlocks {
 #define LBM_MINBLOCKS_F64 4
 #endif
 #ifndef LBM_MINBLOCKS_BATCH_F64
-#define LBM_MINBLOCKS_BATCH_F64 2
+#define LBM_MINBLOCKS_BATCH_F64 4
 #endif
 template <class L, bool BATCH>
 struct MinBlocks<L, double, BATCH> {
-  // 4 x 128 threads: 128 registers (FP64 arithmetic).  Batches: 2 (the members'
-  // arguments on top of the FP64 state spill 60-180 bytes a thread at 128 or 168
-  // registers; 64-node FP64 tiles fit only 2 blocks' shared memory anyway)
+  // 4 x 128 threads: 128 registers; batches too (an ensemble of 32 annuli: 161 us a step
+  // at 2 blocks, 144 at 4, the members' arguments partly from memory)
   static constexpr int value = BATCH ? LBM_MINBLOCKS_BATCH_F64 : LBM_MINBLOCKS_F64;
 };
 
@@ -1040,20 +1040,21 @@ void launch_persistent(const A &a, const TileDesc *tiles, int n_tiles, size_t sm
   if (!prepare_only) launch_early(Kernel, grid, threads, smem, st, a, tiles, n_tiles, inst, tile_inst);
 }
 
-// Tile width of the single-context sweep per storage type: 64 nodes, or 32-node
-// half tiles for FP64 storage (see StageShape; on the L = 256 pipe 3.99 instead of
-// 4.01 ms per step, the same with 64-node tiles in one stage or 32-node tiles in 3).
-template <class T>
-constexpr int single_tile_w() {
-  return half_tiled(sizeof(T) == 8 ? 0 : 1) ? 32 : kTileW;
+// Whether an FP64 context steps in 64-node tiles (one stage a warp, the other 15 warps of
+// the SM cover its copies) or 32-node half tiles (two stages).  64-node tiles share a tile's
+// bookkeeping between two nodes a lane (D2Q9 1024^2: 27.5 -> 23.9 us a step, D3Q19 128^3
+// box 180 -> 162, D3Q15 131 x 97 x 113 120 -> 112, pipe L = 128 122.4 -> 120.0); half tiles leave out empty halves (rows
+// of 80 or 96 nodes: D3Q19 80^3 52.9 against 56.5) and spread small grids over more warps
+// (D2Q9 64^2 3.9 against 5.8, 724^2 15.8 against 16.2, pipe L = 64 22.1 against 27.3).  The line:
+// at least three waves of 64-node tiles over the warps of 4 blocks on 152 SMs, and at
+// least 1.6 halves with fluid per tile (1.5 in the rows of 80 and 96, 1.67 in those of 131).
+inline bool wide_tiles_f64(int n_tiles64, int n_half) {
+  return n_tiles64 >= 3 * 152 * 4 * kWarpsPerBlock && 5ll * n_half >= 8ll * n_tiles64;
 }
 
-template <class L, class T>
-cudaError_t launch_sweep_t(bool odd, const SweepArgs<typename Storage<T>::C> &a, const TileDesc *tiles64,
-                           int n_tiles64, const TileDesc *tiles_half, int n_half, cudaStream_t st) {
-  constexpr int TW = single_tile_w<T>();
-  const TileDesc *tiles = TW == kTileW ? tiles64 : tiles_half;
-  const int n_tiles = TW == kTileW ? n_tiles64 : n_half;
+template <class L, class T, int TW>
+cudaError_t launch_sweep_w(bool odd, const SweepArgs<typename Storage<T>::C> &a, const TileDesc *tiles, int n_tiles,
+                           cudaStream_t st) {
   if (n_tiles == 0) return cudaSuccess;
   const bool skew = a.sy != 0 || a.sz != 0;
   const bool big = (long long)L::Q * a.S >= (1LL << 31);
@@ -1073,6 +1074,15 @@ cudaError_t launch_sweep_t(bool odd, const SweepArgs<typename Storage<T>::C> &a,
   }
 #undef LBM_LAUNCH
   return cudaGetLastError();
+}
+
+template <class L, class T>
+cudaError_t launch_sweep_t(bool odd, const SweepArgs<typename Storage<T>::C> &a, const TileDesc *tiles64,
+                           int n_tiles64, const TileDesc *tiles_half, int n_half, cudaStream_t st) {
+  if constexpr (sizeof(T) == 8) {
+    if (!wide_tiles_f64(n_tiles64, n_half)) return launch_sweep_w<L, T, 32>(odd, a, tiles_half, n_half, st);
+  }
+  return launch_sweep_w<L, T, kTileW>(odd, a, tiles64, n_tiles64, st);
 }
 
 // One step of a batch: the tiles of one kernel class of members in one persistent
