@@ -627,37 +627,36 @@ __device__ __forceinline__ LinkCoef<C> load_coef_nc(const LinkCoef<C> *p) {
   return c;
 }
 
-// Resident blocks per SM the register budget is sized for (launch bounds).  With
-// 4- and 2-byte storage a block of a single-context sweep takes 44.5 KB (D3Q19),
-// 35.8 KB (D3Q15) or 22.5 KB (D2Q9) of shared memory, so 5, 6 or 9 fit an SM: the
-// register budget follows (96, 80 and 64 registers a thread, 5, 6 and 8 blocks).
-// Batch sweeps read their members' arguments from memory into registers: D2Q9 keeps
-// 96 registers (below that it spills, which costs more than the occupancy gains), the
-// 3D lattices take 128 (4 blocks): with 96 they spill 40-200 bytes a thread, and a
-// D3Q19 batch of tilted pipes runs 9 % faster at 4 blocks without spills than at 5
-// with them.
+// Resident blocks per SM the register budget is sized for (launch bounds), each value the
+// fastest of those around it (us a step, smaller / chosen / larger where measured):
+//   D3Q19 FP32 5 (96 registers)      pipe L = 256: 282 / 274 / 276 at 4, 5, 6
+//   D3Q19 16-bit 6                   pipe L = 192 BF16: 112 / 109 / 117 at 5, 6, 7
+//   D3Q15 FP32 5                     131x97x113: 41.5 / 40.2 / 42.1, pipe L = 256: 225 / 215 / 217 at 4, 5, 6
+//   D3Q15 16-bit 6                   pipe L = 192 BF16: 92 / 89 at 5, 6 (131x97x113 FP16: 38 / 40)
+//   D2Q9 8                           2048^2: 29.2 / 29.2 / 29.6 at 7, 8, 9
+// Batch sweeps read their members' arguments from memory into registers:
+//   D2Q9 7                           32 annuli FP32: 58.3 / 57.5 / 61.6 at 6, 7, 8
+//   D3Q19, D3Q15 5                   8 pipes FP32: 108 / 106 / 125 and 90 / 86 / 93 at 4, 5, 6
 #ifndef LBM_MINBLOCKS_F32
 #define LBM_MINBLOCKS_F32 5
 #endif
 #ifndef LBM_MINBLOCKS_D2Q9
 #define LBM_MINBLOCKS_D2Q9 8
 #endif
-#ifndef LBM_MINBLOCKS_D3Q15
-#define LBM_MINBLOCKS_D3Q15 6
-#endif
-#ifndef LBM_MINBLOCKS_D3Q19_2B
-#define LBM_MINBLOCKS_D3Q19_2B 5
+#ifndef LBM_MINBLOCKS_BATCH_D2Q9
+#define LBM_MINBLOCKS_BATCH_D2Q9 7
 #endif
 #ifndef LBM_MINBLOCKS_BATCH_3D
-#define LBM_MINBLOCKS_BATCH_3D 4
+#define LBM_MINBLOCKS_BATCH_3D 5
+#endif
+#ifndef LBM_MINBLOCKS_2B
+#define LBM_MINBLOCKS_2B 6
 #endif
 template <class L, class T, bool BATCH>
 struct MinBlocks {
   static constexpr int value =
-      BATCH ? (L::Q == 9 ? LBM_MINBLOCKS_F32 : LBM_MINBLOCKS_BATCH_3D)
-            : (L::Q == 9 ? LBM_MINBLOCKS_D2Q9
-                         : (L::Q == 15 ? LBM_MINBLOCKS_D3Q15
-                                       : (sizeof(T) == 2 ? LBM_MINBLOCKS_D3Q19_2B : LBM_MINBLOCKS_F32)));
+      BATCH ? (L::Q == 9 ? LBM_MINBLOCKS_BATCH_D2Q9 : LBM_MINBLOCKS_BATCH_3D)
+            : (L::Q == 9 ? LBM_MINBLOCKS_D2Q9 : (sizeof(T) == 2 ? LBM_MINBLOCKS_2B : LBM_MINBLOCKS_F32));
 };
 #ifndef LBM_MINBLOCKS_F64
 #define LBM_MINBLOCKS_F64 4
