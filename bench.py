@@ -52,9 +52,9 @@ WORKLOAD = ("D3Q19 MRT body-force Poiseuille flow in a tilted periodic pipe, L=2
 SCHEME = (0.0, 1.0, 0.0, 1.0)
 BYTES = {"f64": 8, "f32": 4, "bf16": 2, "f16": 2}
 PROFILE = os.path.join(ROOT, "profiles", "sweep_d3q19_f32_pipe192.txt")
-PROFILE_F64 = os.path.join(ROOT, "profiles", "sweep_d3q19_f64_ops_pipe128.txt")
+PROFILE_F64 = os.path.join(ROOT, "profiles", "sweep_d3q19_f64_pipe192.txt")
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_1712_08288_gb300", "csrc", f)
-                  for f in ("sweep.cuh", "common.cuh", "lattice.h", "lbm_internal.h")]
+                  for f in ("sweep.cuh", "common.cuh", "fixed.cuh", "moments.cuh", "lattice.h", "lbm_internal.h")]
 
 
 def kernel_hash():
@@ -89,15 +89,8 @@ def profiled_traffic():
     return _profile_field(PROFILE, "dram_bytes_per_launch_full_size")
 
 
-def profiled_fp64_flops():
-    """FP64 operations per fluid-node update of the FP64 sweep (ncu: DADD + DMUL +
-    2 DFMA thread instructions per launch over the fluid nodes)."""
-    return _profile_field(PROFILE_F64, "fp64_flops_per_fluid_node")
-
-
 def profiled_fp64_instructions():
-    """FP64 pipe instructions (DADD + DMUL + DFMA) per fluid-node update of the FP64
-    sweep (same ncu summary)."""
+    """Instructions on the FP64 pipe per fluid-node update of the FP64 sweep (ncu summary)."""
     return _profile_field(PROFILE_F64, "fp64_instructions_per_fluid_node")
 
 
@@ -281,28 +274,18 @@ def run_gpu(args):
                   "bytes_per_node": 2 * Q * BYTES[prec], "achieved_GBs": round(gbs, 1),
                   "frac_of_hbm": round(gbs / hbm, 4)}
         if prec == "f64":
-            # the FP64 sweep is bound by the FP64 pipe on this GPU: report it against
-            # the measured FMA rate, with the FP64 operations per fluid node counted
-            # by ncu on the same kernel (profiles/)
+            # the collision runs on integers; the FP64 pipe carries conversions and boundary
+            # values: its instructions per second (per fluid node, counted by ncu on the
+            # same kernel, profiles/) against the probe's issue rate (half its flop rate)
             from paper_1712_08288_gb300 import binding as B
             fp64_peak = B.probe_fp64_rate()
-            fl_per_node = profiled_fp64_flops()
             line_p["fp64_peak_gflops"] = round(fp64_peak, 1)
-            if fl_per_node:
-                ach_fl = fl_per_node * n_fluid / (lm * 1e-3) / 1e9
-                line_p["roofline"] = {"bound": "fp64", "flops_per_node": fl_per_node,
-                                      "achieved_gflops": round(ach_fl, 1),
-                                      "frac_of_fp64_peak": round(ach_fl / fp64_peak, 4)}
-                # the FP64 pipe issues one DADD, DMUL or DFMA per slot: the sweep's FP64
-                # instructions per second against the probe's DFMA issue rate (half its
-                # flop rate)
-                in_per_node = profiled_fp64_instructions()
-                if in_per_node:
-                    ach_in = in_per_node * n_fluid / (lm * 1e-3) / 1e9
-                    line_p["roofline"].update({
-                        "fp64_instructions_per_node": in_per_node,
-                        "achieved_ginst_per_s": round(ach_in, 1),
-                        "frac_of_fp64_issue_rate": round(ach_in / (fp64_peak / 2), 4)})
+            in_per_node = profiled_fp64_instructions()
+            if in_per_node:
+                ach_in = in_per_node * n_fluid / (lm * 1e-3) / 1e9
+                line_p["roofline"] = {"bound": "issue", "fp64_instructions_per_node": in_per_node,
+                                      "achieved_ginst_per_s": round(ach_in, 1),
+                                      "frac_of_fp64_issue_rate": round(ach_in / (fp64_peak / 2), 4)}
         prec_lines[prec] = line_p
         del sim
     mlups64 = prec_lines["f64"]["mlups"]
@@ -424,7 +407,6 @@ def summary(line):
     pr = line.get("precisions") or {}
     out = {"frac_hbm": {p: g(pr, p, "frac_of_hbm") for p in ("f32", "bf16", "f16", "f64")},
            "mlups": {p: g(pr, p, "mlups") for p in ("f32", "bf16", "f16", "f64")},
-           "f64_frac_of_fp64_peak": g(pr, "f64", "roofline", "frac_of_fp64_peak"),
            "f64_frac_of_fp64_issue_rate": g(pr, "f64", "roofline", "frac_of_fp64_issue_rate")}
     acc = line.get("accuracy")
     if acc:

@@ -319,8 +319,8 @@ const char *lbm_batch_last_error(const lbm_batch *batch);
 /* The current device's FP64 fused multiply-add rate in GFLOP/s (an FMA counted as
  * two operations), measured with a plain timed FMA loop (8 independent chains per
  * thread, every SM full).  There is no counterpart in the paper: it is the
- * denominator against which the FP64 sweep, bound by the FP64 pipe rather than by
- * HBM on this GPU, is reported.  Runs on the legacy stream and synchronises it;
+ * denominator for what runs on the FP64 pipe, which this GPU has far less of than of
+ * HBM bandwidth.  Runs on the legacy stream and synchronises it;
  * changes no device setting.  LBM_EINVAL for a NULL pointer, LBM_ECUDA if a CUDA
  * call fails. */
 int lbm_probe_fp64_rate(double *gflops);

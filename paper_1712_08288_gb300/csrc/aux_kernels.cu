@@ -33,7 +33,7 @@ __global__ void init_eq_kernel(AuxArgs a, const double *rho, const double *u) {
     }
     // Eq. 42 minus w_i rho0, c_s^2 = 1/3: w_i (drho + rho0 (3 c + 4.5 c^2 - 1.5 u^2)) with c =
     // e_i.u, the even part shared by a direction and its opposite (FP64 instructions are
-    // what this kernel costs: 128^3 D3Q19 455 -> 280 us)
+    // what this kernel costs: 128^3 D3Q19 455 -> 266 us)
     const double A = drho - 1.5 * a.rho0 * (ux * ux + uy * uy + uz * uz);
     Storage<T>::store(pop + n, L::w(0) * A);
 #pragma unroll

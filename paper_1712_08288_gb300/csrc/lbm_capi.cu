@@ -423,7 +423,7 @@ static int upload_tiles(lbm_ctx *c, const uint8_t *solid, const std::vector<uint
   t.d.reserve((size_t)nxb * c->ny * c->nz);
   std::vector<uint32_t> rec32;
   std::vector<uint16_t> ldesc;
-  if (bmask) rec32.reserve(bmask->size());
+  if (bmask && !per_link(c->precision)) rec32.reserve(bmask->size());
   if (with_links) ldesc.reserve((size_t)c->n_links);
   int rb = 0;
   for (int z = 0; z < c->nz; ++z)
@@ -452,7 +452,7 @@ static int upload_tiles(lbm_ctx *c, const uint8_t *solid, const std::vector<uint
                 ldesc.push_back((uint16_t)((k & 31) | (__builtin_ctz(w) << kLinkDirShift)));
             }
             d.bnd |= 1ull << k;
-            rec32.push_back(m | ((off - (uint32_t)d.lb) << kRecShift));
+            if (!with_links) rec32.push_back(m | ((off - (uint32_t)d.lb) << kRecShift));
             ++rb;
           }
         }

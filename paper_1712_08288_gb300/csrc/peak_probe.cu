@@ -1,6 +1,5 @@
 // peak_probe.cu -- lbm_probe_fp64_rate: the device's FP64 fused multiply-add rate,
-// measured with a plain FMA loop, the denominator the FP64 sweep (bound by the
-// FP64 pipe on this GPU, not by HBM) is reported against.  No device setting is
+// measured with a plain FMA loop, the denominator for what runs on the FP64 pipe.  No device setting is
 // changed; the probe allocates 8 bytes and frees them.
 #include <cuda_runtime.h>
 
