@@ -17,10 +17,14 @@ namespace lbm {
 //
 // The adjoint populations are multiples of 2^(E_l - 53), E_l their largest exponent; sums
 // with M (up to 192 times the largest) fit 62 bits.  Scaled moments and results are
-// multiples of 2^(E_l - 57).  For every s in [0, 2] and |u_a| < 0.63 (deviations under rho0/16,
-// fx_block's range) results stay below 13 times the largest adjoint value and the sums in
-// fx_meq_adjoint below 8 times (row sums of the transposed operator): 62 bits.  Nodes
-// outside these ranges take the FP64 form.
+// multiples of 2^(E_l - 57), the largest adjoint value is below 2^58 of them, and 64 bits
+// hold 32 times that.  For every s in [0, 2] and |u_a| < 0.63 (deviations under rho0/16,
+// fx_block's range) results stay below 13 times the largest adjoint value and the factors of the
+// velocity in fx_meq_adjoint below 8 times (row sums of the transposed operator).  Rows e
+// and eps of D3Q19 arrive 8 and 4 times larger: the sums with them stay below 24.4 times
+// before their shifts (a in fx_meq_adjoint: 19 x 8 x 2 x 192 / 2394 at s_e = 2, s_eps = 0;
+// 38 and 22 for its factors, with a shift by 3, would reach 48.8).  tests/test_fixed_point_host.py
+// runs the extremes with overflow checks.  Nodes outside these ranges take the FP64 form.
 // ---------------------------------------------------------------------------
 constexpr int kAdjIn = 53, kAdjOut = 57;
 template <class L>
@@ -89,7 +93,7 @@ LBM_HD void fx_meq_adjoint(D3Q15, const i64 (&smu)[15], FxHalves ux, FxHalves uy
 LBM_HD void fx_meq_adjoint(D3Q19, const i64 (&smu)[19], FxHalves ux, FxHalves uy, FxHalves uz,
                            i64 (&out)[4]) {
   out[0] = (6 * smu[2] - 11 * smu[1] + 4) >> 3;              // -11/8, 3/4
-  const i64 a = (38 * smu[1] - 22 * smu[2] + 4) >> 3;        // 38/8, -11/4
+  const i64 a = (19 * smu[1] - 11 * smu[2] + 2) >> 2;        // 38/8, -11/4
   const i64 yz = a - 2 * smu[9] + smu[10], w = 2 * smu[11] - smu[12];
   out[1] = adj_times(a + 4 * smu[9] - 2 * smu[10], ux) + adj_times(smu[13], uy) + adj_times(smu[15], uz);
   out[2] = adj_times(yz + w, uy) + adj_times(smu[13], ux) + adj_times(smu[14], uz);
