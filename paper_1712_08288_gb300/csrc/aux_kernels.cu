@@ -168,7 +168,6 @@ __global__ void __launch_bounds__(kNormThreads, 3)
     const int k = threadIdx.x;
     double v = sh[0][k];
     for (int w = 1; w < kNormThreads / 32; ++w) v = (k == 2) ? fmax(v, sh[w][k]) : v + sh[w][k];
-    if (k >= 4 && k <= 6) v *= momentum_factor(a);
     partials[(long long)blockIdx.x * kNormFields + k] = v;
   }
 }

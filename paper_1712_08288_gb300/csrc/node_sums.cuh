@@ -9,8 +9,8 @@
 // 32-bit and 16-bit storage: every population within 2^33 of the largest is exact, so the
 // sums are too; smaller ones lose less than 2^-57 of the largest.  FP64 storage: one unit
 // is 1/32 of an ulp of the largest population, where an FP64 sum rounds each
-// addition.  Nodes with a non-finite value, or with none above the small end of
-// the range, take FP64 sums.
+// addition.  Nodes with a non-finite value, with none above the small end of the range, or
+// with one so large that a sum could leave the range of FP64, take FP64 sums.
 #pragma once
 
 #include "common.cuh"
@@ -64,29 +64,34 @@ __device__ __forceinline__ void load_node(typename Storage<T>::C (&g)[L::Q], int
   }
 }
 
-// rho - rho0 and j / rho0 of a node, and j in the form that sums add up: j / rho0 where
-// rho0 is a power of two (exact), j otherwise (momentum_factor() undoes it)
+// rho - rho0, j / rho0 and j of a node
 struct NodeSums {
   double drho, u[3], j[3];
 };
-__device__ __forceinline__ double momentum_factor(const AuxArgs &a) {
-  return a.rho0_exp != AuxArgs::kNoPowerOfTwo ? a.rho0 : 1.0;
-}
 
-// Sums of the integers times 2^scale.  A power of two rho0 divides j exactly through the
-// exponents (AuxArgs::rho0_exp), at no cost.
+// Sums of the integers times 2^scale, by adding to the exponent of the converted sum:
+// the caller has checked that scale (and scale - rho0_exp) keeps every sum of 1 to 2^63
+// units within the exponents of normal numbers.  A power of two rho0 divides j exactly
+// through the exponents (AuxArgs::rho0_exp), at no cost.
 template <class L>
 __device__ __forceinline__ NodeSums scaled_sums(const i64 (&v)[L::Q], int scale, const AuxArgs &a) {
   i64 m[L::Q];
   fmoments<i64>(L{}, v, m);   // rho and j are used, the rest is never computed
-  auto to = [&](i64 x, int sc) {
-    const double d = (double)x;
-    return __hiloint2double(x != 0 ? __double2hiint(d) + (sc << 20) : 0, __double2loint(d));
+  auto times = [&](double d, int sc) {
+    const int hi = __double2hiint(d);      // 0 only for d = 0
+    return __hiloint2double(hi != 0 ? hi + (sc << 20) : 0, __double2loint(d));
   };
   const bool two = a.rho0_exp != AuxArgs::kNoPowerOfTwo;
+  const double x = (double)m[3], y = (double)m[5], z = L::D == 3 ? (double)m[7] : 0.0;
+  NodeSums r;
+  r.drho = times((double)m[0], scale);
+  r.j[0] = times(x, scale);
+  r.j[1] = times(y, scale);
+  r.j[2] = times(z, scale);
   const int su = two ? scale - a.rho0_exp : scale;
-  const double x = to(m[3], su), y = to(m[5], su), z = L::D == 3 ? to(m[7], su) : 0.0;
-  NodeSums r = {to(m[0], scale), {x, y, z}, {x, y, z}};
+  r.u[0] = times(x, su);
+  r.u[1] = times(y, su);
+  r.u[2] = times(z, su);
   if (!two) {
 #pragma unroll
     for (int k = 0; k < L::D; ++k) r.u[k] /= a.rho0;
@@ -105,12 +110,7 @@ __device__ __forceinline__ NodeSums plain_sums(const C (&g)[L::Q], const AuxArgs
     if (L::ey(i) != 0) j[1] += L::ey(i) * v;
     if (L::ez(i) != 0) j[2] += L::ez(i) * v;
   }
-  NodeSums r = {drho, {j[0] / a.rho0, j[1] / a.rho0, j[2] / a.rho0}, {j[0], j[1], j[2]}};
-  if (a.rho0_exp != AuxArgs::kNoPowerOfTwo) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) r.j[k] = r.u[k];
-  }
-  return r;
+  return {drho, {j[0] / a.rho0, j[1] / a.rho0, j[2] / a.rho0}, {j[0], j[1], j[2]}};
 }
 
 template <class L>
@@ -142,7 +142,9 @@ __device__ __forceinline__ NodeSums node_sums(const double (&g)[L::Q], const Aux
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) mx = max(mx, __double2hiint(g[i]) & 0x7fffffff);
   const int E = mx >> 20;
-  if (mx != 0 && (E < kFxMinExp || E == 2047)) return plain_sums<L>(g, a);
+  // exponents of the sums' units, over rho0 too where that is a shift: see scaled_sums()
+  const int Eu = a.rho0_exp != AuxArgs::kNoPowerOfTwo ? E - a.rho0_exp : E;
+  if (mx != 0 && (min(E, Eu) < kFxMinExp || max(E, Eu) > 1900)) return plain_sums<L>(g, a);
   i64 v[L::Q];
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) v[i] = fx_from<kTop>(g[i], max(E, kFxMinExp));
