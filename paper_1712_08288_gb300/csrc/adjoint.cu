@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(kAdjThreads, sizeof(C) == 4 ? 6 : 3)
   }
 }
 
-// add the per-link sums of one segment to the FP64 totals and clear them
+// add the per-link sums of the last steps to the FP64 totals and clear them
 template <class C>
 __global__ void link_flush_kernel(C *acc, double *tot, long long n) {
   wait_for_previous();

@@ -1205,6 +1205,11 @@ int adjoint_backward_impl(lbm_ctx *c, double *grad_s, double *grad_q, double *gr
   // when an earlier backward pass has overwritten the states the forward pass left),
   // then step back through it
   char *lin = lam0, *lout = lam1;
+  // The links' sums are held in the compute type and added to the FP64 totals after every
+  // segment and at least every sqrt(T) steps: with every state kept the run is one segment,
+  // and sequential FP32 sums over 20000 steps would keep 5 digits instead of 7.
+  const long long flush_every = (long long)std::ceil(std::sqrt((double)T));
+  long long unflushed = 0;
   const bool last_saved = tp.last_saved;
   tp.last_saved = last_saved && nseg == 1;   // a recomputation below reuses the segment buffer
   for (long long sgm = nseg - 1; sgm >= 0; --sgm) {
@@ -1233,8 +1238,11 @@ int adjoint_backward_impl(lbm_ctx *c, double *grad_s, double *grad_q, double *gr
       ADJ_CUDA(launch_adjoint_step(c->lattice, c->precision, c->a64, c->a32, aux_args(c), dcoef,
                                    acc, at(r), lin, lout, gpart, st));
       std::swap(lin, lout);
+      if (++unflushed == flush_every || r == 0) {
+        ADJ_CUDA(launch_link_flush(c->precision, acc, dtot, 2 * nl, st));
+        unflushed = 0;
+      }
     }
-    ADJ_CUDA(launch_link_flush(c->precision, acc, dtot, 2 * nl, st));
   }
   ADJ_CUDA(launch_adjoint_finish(c->lattice, gpart, pblocks, dgs, st));
   // back to the state after the forward run
