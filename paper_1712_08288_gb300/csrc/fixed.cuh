@@ -23,9 +23,11 @@
 // Range.  The bounds below hold for deviations under rho0/16 (and under 2^15, where a
 // density cannot pass the runaway limit of 1e6); a node outside that range, with a
 // non-finite entry, or with all entries under 2^-895 takes the FP64 form, so any input
-// gives what it gave (values that all lie below 2^-1042 count as a node at rest).  With g the largest deviation, |j_a| <= 10 g and j_a j_b / rho0 <= 6.3 g (D2Q9:
-// 6 g and 2.3 g), every sum given to fx_mul is below 45 g (D2Q9: 25 g) and every result
-// below 55 g (D2Q9: 16 g): all within 64 bits.
+// gives what it gave (values that all lie below 2^-1042 count as a node at rest), and so
+// do contexts without a relaxed row (every s_k = 0), whose advection is exact.  With g the
+// largest deviation, |j_a| <= 10 g and j_a j_b / rho0 <= 6.3 g (D2Q9: 6 g and 2.3 g), every
+// sum given to fx_mul is below 45 g (D2Q9: 25 g) and every result below 55 g (D2Q9: 16 g):
+// all within 64 bits.
 #pragma once
 
 #include <math.h>
@@ -328,7 +330,10 @@ inline FixedArgs fx_args(const double *s, double rho0, const double *F) {
   fx.inv_rho0 = fx_coef(mr / 4);
   fx.quad_shift = kFxTop<L> + 963 - er;
   fx.max_exp = 1023 + (ilogb(rho0) - 5 < 14 ? ilogb(rho0) - 5 : 14);
-  if (fx.max_exp < kFxMinExp) fx.max_exp = -1;
+  // no relaxed row: the populations move on unchanged, which the FP64 form does bit for bit
+  bool relaxes = false;
+  for (int k = 0; k < L::Q; ++k) relaxes |= !L::conserved(k) && s[k] != 0.0;
+  if (fx.max_exp < kFxMinExp || !relaxes) fx.max_exp = -1;
   fx.force_hi = 0;
   for (int a = 0; a < 3; ++a)
     if ((fx_hi(F[a]) & 0x7fffffff) > fx.force_hi) fx.force_hi = fx_hi(F[a]) & 0x7fffffff;
