@@ -243,8 +243,9 @@ int lbm_set_link_values(lbm_ctx *ctx, const double *q, const double *uw);
  *   J = sum over fluid nodes n with mask[n] != 0 of |u(x_n, T) - u_target(x_n)|^2,
  * u the reported velocity after the n_steps (T = current time + n_steps).
  * The forward run keeps a checkpoint every checkpoint_every steps (0 = every state of
- * the run where they take at most 4 GiB and 1/16 of the free memory, else about
- * sqrt(n_steps)); the backward pass recomputes one segment at a time from its
+ * the run where they take at most 4 GiB and 1/16 of the free memory, and all contexts
+ * that keep theirs at most 1/16 of the device's memory, else about sqrt(n_steps); pass a
+ * value where the memory must not depend on that); the backward pass recomputes one segment at a time from its
  * checkpoint and runs the adjoint sweep through it.  The last segment, or the only
  * one, keeps its states and is not recomputed.  On return the context is in
  * the state after the forward run (as if lbm_step(n_steps) had been called).
@@ -257,8 +258,9 @@ int lbm_set_link_values(lbm_ctx *ctx, const double *q, const double *uw);
  * The adjoint computes in double for LBM_F64 and in float otherwise; gradients
  * are accumulated in double (a link's, from sums over at most sqrt(n_steps) steps in
  * the compute type).  Memory: about (n_steps/checkpoint_every +
- * checkpoint_every + 3) population arrays, kept in the context after a successful
- * call and reused (grown when needed) by later calls; lbm_destroy releases it. */
+ * checkpoint_every + 3) population arrays, n_steps + 3 where every state is kept,
+ * held in the context after a successful call and reused (grown when needed) by later
+ * calls; lbm_destroy releases it. */
 int lbm_adjoint(lbm_ctx *ctx, int n_steps, int checkpoint_every, const uint8_t *mask,
                 const double *u_target, double *loss, double *grad_s, double *grad_q,
                 double *grad_uw);

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -109,6 +110,7 @@ struct lbm_ctx {
   std::vector<int64_t> link_src; // input position of the link at each device position
   // device workspace of lbm_adjoint (pointer, capacity), kept between calls
   std::pair<void *, size_t> adj_ws[13] = {};
+  size_t adj_kept = 0;          // part of it that counts towards the device's kept states
   AdjTape tape;                 // what lbm_adjoint_forward left for the backward pass
   long long state_serial = 0;   // bumped by every call that changes the populations
   long long n_links = 0, n_fluid = 0, n_boundary = 0;
@@ -298,8 +300,16 @@ static cudaError_t adj_ws_get(lbm_ctx *c, int slot, size_t bytes, void **p) {
   *p = e.first;
   return cudaSuccess;
 }
+// Bytes that contexts of a device hold because their adjoint runs kept every state (see
+// keep_every_state), all contexts of the process together.
+constexpr int kKeptDevices = 64;
+static std::atomic<size_t> g_adj_kept[kKeptDevices];
+static std::atomic<size_t> &adj_kept_on(int device) { return g_adj_kept[(unsigned)device % kKeptDevices]; }
+
 static void adj_ws_free(lbm_ctx *c) {
   c->tape.valid = false;
+  adj_kept_on(c->device) -= c->adj_kept;
+  c->adj_kept = 0;
   for (auto &e : c->adj_ws) {
     cudaFree(e.first);
     e = {nullptr, 0};
@@ -1008,16 +1018,25 @@ enum AdjSlot { kCk = 0, kSeg, kFin, kLam0, kLam1, kMask, kUt, kGs, kTot, kAcc, k
 // Whether a run of T steps keeps every state instead of checkpoints (checkpoint_every =
 // 0).  The forward sweep then writes each state once (half a step's traffic more) and the
 // backward pass recomputes nothing (a whole step's traffic less, and a launch).  Limits:
-// 4 GiB in all -- sqrt(T) checkpoints of a run of that length take up to a few GiB
-// themselves -- and, where the workspace has to grow for it, 1/16 of the free memory.
+// 4 GiB a context -- sqrt(T) checkpoints of a run of that length take up to a few GiB
+// themselves --, 1/16 of the device's memory for all contexts together (they hold it until
+// they are destroyed), and, where the workspace has to grow for it, 1/16 of the free memory.
 // D3Q19 FP32, 64^3 x 144 steps (2.9 GB), forward and backward: 6.7 -> 4.8 ms.
 constexpr size_t kKeepAllBytes = (size_t)4 << 30;
-bool keep_every_state(const lbm_ctx *c, long long T, size_t state) {
+bool keep_every_state(lbm_ctx *c, long long T, size_t state) {
   if (state == 0 || (size_t)T > kKeepAllBytes / state) return false;
   const size_t all = state * (size_t)T, have = c->adj_ws[kSeg].second;
   if (have >= all) return true;
   size_t free_b = 0, total_b = 0;
-  return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && all - have <= free_b / 16;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || all - have > free_b / 16) return false;
+  std::atomic<size_t> &kept = adj_kept_on(c->device);
+  const size_t more = all - std::min(all, c->adj_kept);
+  size_t now = kept.load();
+  do {
+    if (now + more > total_b / 16) return false;
+  } while (!kept.compare_exchange_weak(now, now + more));
+  c->adj_kept += more;
+  return true;
 }
 
 int adjoint_forward_impl(lbm_ctx *c, int n_steps, int checkpoint_every, const uint8_t *mask,
