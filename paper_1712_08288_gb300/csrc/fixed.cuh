@@ -8,8 +8,11 @@
 // two integer instructions and exact.  D3Q19, 32 nodes on one SM: 3413 cycles in FP64, 471
 // here (1216 instructions, 19 of them conversions on the FP64 pipe); D2Q9 1364 and 212.
 // The D3Q19 pipe at L = 128: 546 us a step in FP64, 164 with this collision alone.  Error
-// of a step against quad precision, rms in half ulps of the node's largest deviation,
-// FP64 and here: D2Q9 0.26 and 0.24, D3Q15 0.47 and 0.32, D3Q19 0.49 and 0.31.
+// of a step against extended precision, rms in half ulps of the node's largest deviation
+// (rounding the result once is 0.28 to 0.33 of that), FP64 form with fused multiply-adds and
+// here, at s_nu 0.5 to 1.9 and the workloads' other rates: D2Q9 0.45-0.77 and 0.34-0.36,
+// D3Q15 0.41-0.61 and 0.37-0.40, D3Q19 0.68-0.73 and 0.38-0.44.  Where every rate is far below
+// 1 the FP64 form subtracts little and rounds little: all rates 0.05, D3Q15 0.28 and 0.43.
 //
 // Number form.  With E the largest exponent among the node's deviations and the force,
 // value = v 2^(E - top) with top = 56 (57 for D2Q9): the largest |v| is below 2^(top+1),

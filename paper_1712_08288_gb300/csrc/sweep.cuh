@@ -41,7 +41,7 @@ namespace lbm {
 // al. 2002 for D3Q19 with w_eps = 3, w_epsj = -11/2, w_xx = -1/2; the Appendix's
 // D3Q15 basis below).
 template <class C>
-__device__ __forceinline__ C meq(D2Q9, int k, C drho, C jx, C jy, C, C ir0) {
+LBM_HD C meq(D2Q9, int k, C drho, C jx, C jy, C, C ir0) {
   switch (k) {
     case 1: return C(-2) * drho + C(3) * (jx * jx + jy * jy) * ir0;
     case 2: return drho - C(3) * (jx * jx + jy * jy) * ir0;
@@ -53,7 +53,7 @@ __device__ __forceinline__ C meq(D2Q9, int k, C drho, C jx, C jy, C, C ir0) {
   }
 }
 template <class C>
-__device__ __forceinline__ C meq(D3Q19, int k, C drho, C jx, C jy, C jz, C ir0) {
+LBM_HD C meq(D3Q19, int k, C drho, C jx, C jy, C jz, C ir0) {
   const C j2 = (jx * jx + jy * jy + jz * jz) * ir0;
   switch (k) {
     case 1: return C(-11) * drho + C(19) * j2;
@@ -75,7 +75,7 @@ __device__ __forceinline__ C meq(D3Q19, int k, C drho, C jx, C jy, C jz, C ir0) 
 // D3Q15 (Appendix basis): e^eq = -rho + j^2/rho0, eps^eq = rho - 5 j^2/rho0,
 // q^eq = -7/3 j, second-order rows j_a j_b / rho0 combinations, m_xyz^eq = 0
 template <class C>
-__device__ __forceinline__ C meq(D3Q15, int k, C drho, C jx, C jy, C jz, C ir0) {
+LBM_HD C meq(D3Q15, int k, C drho, C jx, C jy, C jz, C ir0) {
   const C j2 = (jx * jx + jy * jy + jz * jz) * ir0;
   switch (k) {
     case 1: return -drho + j2;
@@ -131,8 +131,7 @@ __device__ __forceinline__ C madd(C acc, int m, C v) {
 // edge and face parts and the plane parts.  Same operator as the generic pair form
 // below, with about a third fewer operations; rounding order differs.
 template <class C>
-__device__ __forceinline__ void collide_d3q19(const C (&g)[19], C (&gp)[19], const SweepArgs<C> &a,
-                                              C &drho_out) {
+LBM_HD void collide_d3q19(const C (&g)[19], C (&gp)[19], const SweepArgs<C> &a, C &drho_out) {
   C s[9], d[9];
 #pragma unroll
   for (int p = 0; p < 9; ++p) {
@@ -213,8 +212,7 @@ __device__ __forceinline__ void collide_d3q19(const C (&g)[19], C (&gp)[19], con
 // / |M_k|^2 on the relaxed rows, r = -F on the momentum rows (the force term), and
 // g' = g - M^T r.
 template <class L, class C>
-__device__ __forceinline__ void collide_factored(const C (&g)[L::Q], C (&gp)[L::Q], const SweepArgs<C> &a,
-                                                 C &drho_out) {
+LBM_HD void collide_factored(const C (&g)[L::Q], C (&gp)[L::Q], const SweepArgs<C> &a, C &drho_out) {
   constexpr int Q = L::Q;
   C m[Q];
   fmoments<C>(L{}, g, m);
@@ -232,6 +230,15 @@ __device__ __forceinline__ void collide_factored(const C (&g)[L::Q], C (&gp)[L::
   fmt<false, C>(L{}, r, t);
 #pragma unroll
   for (int i = 0; i < Q; ++i) gp[i] = g[i] - t[i];
+}
+
+// the factored form of the lattice
+template <class L, class C>
+LBM_HD C collide_plain(const C (&g)[L::Q], C (&gp)[L::Q], const SweepArgs<C> &a) {
+  C drho;
+  if constexpr (std::is_same_v<L, D3Q19>) collide_d3q19<C>(g, gp, a, drho);
+  else collide_factored<L, C>(g, gp, a, drho);
+  return drho;
 }
 
 // FP64 storage: the collision in block fixed point (fixed.cuh) where the node's values
@@ -268,10 +275,7 @@ __device__ __forceinline__ bool collide(const C (&g)[L::Q], C (&gp)[L::Q], const
     if (collide_fixed<L>(g, gp, a)) return false;
   }
   if constexpr (sizeof(C) == 8 || sizeof(T) == 2) {
-    C drho;
-    if constexpr (std::is_same_v<L, D3Q19>) collide_d3q19<C>(g, gp, a, drho);
-    else collide_factored<L, C>(g, gp, a, drho);
-    return !(fabs(drho) < C(1e6));
+    return !(fabs(collide_plain<L, C>(g, gp, a)) < C(1e6));
   }
   constexpr int Q = L::Q;
   constexpr int NP = L::NP;

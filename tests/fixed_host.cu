@@ -6,7 +6,7 @@
 // in:  doubles n, rho0, F[3] (the force on the momentum rows), s[19], then per node g[Q]
 //      and, for adjoint, lambda'[Q].
 // out: per node 1.0 where the fixed-point form covers it (else 0.0), then for collide g'[Q]
-//      and Q zeros, for adjoint the transpose t[Q] and dJ/ds[Q].
+//      in fixed point and g'[Q] in FP64, for adjoint the transpose t[Q] and dJ/ds[Q].
 #include <stdio.h>
 #include <string.h>
 
@@ -39,6 +39,7 @@ static int run(bool adjoint) {
         z[k] = L::conserved(k) ? 0.0 : z[k] * -fx_neq_scale<L>(k) / (1 << fx_fine<L>(k));
     } else {
       ok = collide_fixed<L>(g, y, a);
+      collide_plain<L>(g, z, a);
     }
     const double flag = ok ? 1.0 : 0.0;
     put(&flag, 1);
