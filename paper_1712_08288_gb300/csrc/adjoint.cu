@@ -155,45 +155,6 @@ __host__ __device__ constexpr int nc_slot(int k) {
 static_assert(nc_slot<D3Q19>(19) <= 16 && nc_slot<D3Q15>(15) <= 16 && nc_slot<D2Q9>(9) <= 16,
               "at most 16 relaxed rows");
 
-// sum_k smu_k * d meq_k / d(rho, j_x, j_y, j_z) for the equilibrium moments of
-// meq() (deviation form), smu_k = s_k mu_k on the non-conserved rows
-template <class C>
-__device__ __forceinline__ void meq_adjoint(D2Q9, const C (&smu)[9], C jx, C jy, C, C ir0,
-                                            C (&out)[4]) {
-  out[0] = C(-2) * smu[1] + smu[2];
-  const C a = C(6) * (smu[1] - smu[2]) * ir0;
-  out[1] = a * jx - smu[4] + (C(2) * smu[7] * jx + smu[8] * jy) * ir0;
-  out[2] = a * jy - smu[6] + (C(-2) * smu[7] * jy + smu[8] * jx) * ir0;
-  out[3] = C(0);
-}
-template <class C>
-__device__ __forceinline__ void meq_adjoint(D3Q19, const C (&smu)[19], C jx, C jy, C jz, C ir0,
-                                            C (&out)[4]) {
-  out[0] = C(-11) * smu[1] + C(3) * smu[2];
-  const C a = (C(38) * smu[1] - C(11) * smu[2]) * ir0;    // e, eps: 19 j^2, -5.5 j^2
-  const C px = (C(4) * smu[9] - C(2) * smu[10]) * ir0;    // 3p_xx, 3pi_xx along j_x
-  const C pyz = (C(-2) * smu[9] + smu[10]) * ir0;         // 3p_xx, 3pi_xx along j_y, j_z
-  const C w = (C(2) * smu[11] - smu[12]) * ir0;           // p_ww, pi_ww along j_y (-w along j_z)
-  const C c23 = C(2.0 / 3.0);
-  out[1] = (a + px) * jx - c23 * smu[4] + (smu[13] * jy + smu[15] * jz) * ir0;
-  out[2] = (a + pyz + w) * jy - c23 * smu[6] + (smu[13] * jx + smu[14] * jz) * ir0;
-  out[3] = (a + pyz - w) * jz - c23 * smu[8] + (smu[14] * jy + smu[15] * jx) * ir0;
-}
-
-template <class C>
-__device__ __forceinline__ void meq_adjoint(D3Q15, const C (&smu)[15], C jx, C jy, C jz, C ir0,
-                                            C (&out)[4]) {
-  out[0] = -smu[1] + smu[2];
-  const C a = (C(2) * smu[1] - C(10) * smu[2]) * ir0;    // e, eps: j^2, -5 j^2
-  const C px = C(4) * smu[9] * ir0;                      // 3p_xx along j_x
-  const C pyz = C(-2) * smu[9] * ir0;                    // 3p_xx along j_y, j_z
-  const C w = C(2) * smu[10] * ir0;                      // p_ww along j_y (-w along j_z)
-  const C c73 = C(7.0 / 3.0);
-  out[1] = (a + px) * jx - c73 * smu[4] + (smu[11] * jy + smu[13] * jz) * ir0;
-  out[2] = (a + pyz + w) * jy - c73 * smu[6] + (smu[11] * jx + smu[12] * jz) * ir0;
-  out[3] = (a + pyz - w) * jz - c73 * smu[8] + (smu[12] * jy + smu[13] * jx) * ir0;
-}
-
 // One step back in time, one node per thread.  SMALL: node indices fit in 31 bits,
 // so neighbour indices come from the node's wrapped coordinates in 32-bit
 // arithmetic.
@@ -217,7 +178,6 @@ __global__ void __launch_bounds__(kAdjThreads, sizeof(C) == 4 ? LBM_ADJ_MINB_F32
       y = (int)(r % a.ny);
       z = (int)(r / a.ny);
     }
-    const C ir0 = sa.inv_rho0;
     C g[Q], lp[Q], lpre[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -285,36 +245,11 @@ __global__ void __launch_bounds__(kAdjThreads, sizeof(C) == 4 ? LBM_ADJ_MINB_F32
     bool done = false;
     if constexpr (sizeof(C) == 8) done = fx_adjoint<L>(g, lp, sa.fx, ag.fx, t, gsum);
     if (!done) {
-      // the factored transforms (fmoments, fmt): fewer operations than the pair form
-      // (FP32: 0.349 -> 0.340 s for the backward pass at 128^3 x 2000)
-      C m[Q], mu[Q];
-      fmoments<C>(L{}, g, m);
-      fmoments<C>(L{}, lp, mu);
-      const C jx = m[3], jy = m[5], jz = L::D == 3 ? m[7] : C(0);
-      C smu[Q], nu[Q];
-#pragma unroll
-      for (int k = 0; k < Q; ++k) {
-        if (Rows<L>::cons(k)) {
-          smu[k] = C(0);
-          mu[k] *= C(1.0 / row_norm2<L>(k));
-          continue;
-        }
-        smu[k] = sa.sn[k] * mu[k];                                      // s_k (M lambda')_k / |M_k|^2
-        mu[k] *= C(1.0 / row_norm2<L>(k));
-        gsum[k] = mu[k] * (meq(L{}, k, m[0], jx, jy, jz, ir0) - m[k]);   // d m'_k/d s_k
-        nu[k] = mu[k] - smu[k];                                         // (1 - s_k) mu_k
-      }
-      C dq[4];
-      meq_adjoint(L{}, smu, jx, jy, jz, ir0, dq);
-      nu[0] = mu[0] + dq[0];
-      nu[3] = mu[3] + dq[1];
-      nu[5] = mu[5] + dq[2];
-      if (L::D == 3) nu[7] = mu[7] + dq[3];
-      fmt<true, C>(L{}, nu, t);
+      adjoint_plain<L, C>(g, lp, sa, t, gsum);
       if constexpr (sizeof(C) == 8) {
 #pragma unroll
         for (int k = 0; k < Q; ++k)
-          if (!Rows<L>::cons(k)) gsum[k] *= -(1 << fx_fine<L>(k)) / fx_neq_scale<L>(k);
+          if (!Rows<L>::cons(k)) gsum[k] *= 1.0 / fx_gsum_scale<L>(k);
       }
     }
     if constexpr (sizeof(C) == 8) {
@@ -361,7 +296,7 @@ __global__ void __launch_bounds__(kAdjThreads, sizeof(C) == 4 ? LBM_ADJ_MINB_F32
     for (int k = 0; k < Q; ++k)
       if (k == (int)threadIdx.x) {
         slot = nc_slot<L>(k);
-        if constexpr (sizeof(C) == 8) scale = -fx_neq_scale<L>(k) / (1 << fx_fine<L>(k));
+        if constexpr (sizeof(C) == 8) scale = fx_gsum_scale<L>(k);
       }
     C t = C(0);
     for (int w = 0; w < kAdjThreads / 32; ++w) t += sh[w][slot];

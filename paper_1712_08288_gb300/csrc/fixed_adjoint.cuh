@@ -1,11 +1,87 @@
-// fixed_adjoint.cuh -- the transpose of the FP64 collision in block fixed point, for the
-// adjoint step (adjoint.cu); callable on the host too, as fixed.cuh is.
+// fixed_adjoint.cuh -- the transpose of the collision for the adjoint step (adjoint.cu), in
+// the compute type and, for FP64 storage, in block fixed point; callable on the host too,
+// as fixed.cuh is.
 #pragma once
 
 #include "fixed.cuh"
 #include "sweep.cuh"
 
 namespace lbm {
+
+// sum_k smu_k * d meq_k / d(rho, j_x, j_y, j_z) for the equilibrium moments of
+// meq() (deviation form), smu_k = s_k mu_k on the non-conserved rows
+template <class C>
+LBM_HD void meq_adjoint(D2Q9, const C (&smu)[9], C jx, C jy, C, C ir0,
+                        C (&out)[4]) {
+  out[0] = C(-2) * smu[1] + smu[2];
+  const C a = C(6) * (smu[1] - smu[2]) * ir0;
+  out[1] = a * jx - smu[4] + (C(2) * smu[7] * jx + smu[8] * jy) * ir0;
+  out[2] = a * jy - smu[6] + (C(-2) * smu[7] * jy + smu[8] * jx) * ir0;
+  out[3] = C(0);
+}
+template <class C>
+LBM_HD void meq_adjoint(D3Q19, const C (&smu)[19], C jx, C jy, C jz, C ir0,
+                        C (&out)[4]) {
+  out[0] = C(-11) * smu[1] + C(3) * smu[2];
+  const C a = (C(38) * smu[1] - C(11) * smu[2]) * ir0;    // e, eps: 19 j^2, -5.5 j^2
+  const C px = (C(4) * smu[9] - C(2) * smu[10]) * ir0;    // 3p_xx, 3pi_xx along j_x
+  const C pyz = (C(-2) * smu[9] + smu[10]) * ir0;         // 3p_xx, 3pi_xx along j_y, j_z
+  const C w = (C(2) * smu[11] - smu[12]) * ir0;           // p_ww, pi_ww along j_y (-w along j_z)
+  const C c23 = C(2.0 / 3.0);
+  out[1] = (a + px) * jx - c23 * smu[4] + (smu[13] * jy + smu[15] * jz) * ir0;
+  out[2] = (a + pyz + w) * jy - c23 * smu[6] + (smu[13] * jx + smu[14] * jz) * ir0;
+  out[3] = (a + pyz - w) * jz - c23 * smu[8] + (smu[14] * jy + smu[15] * jx) * ir0;
+}
+
+template <class C>
+LBM_HD void meq_adjoint(D3Q15, const C (&smu)[15], C jx, C jy, C jz, C ir0,
+                        C (&out)[4]) {
+  out[0] = -smu[1] + smu[2];
+  const C a = (C(2) * smu[1] - C(10) * smu[2]) * ir0;    // e, eps: j^2, -5 j^2
+  const C px = C(4) * smu[9] * ir0;                      // 3p_xx along j_x
+  const C pyz = C(-2) * smu[9] * ir0;                    // 3p_xx along j_y, j_z
+  const C w = C(2) * smu[10] * ir0;                      // p_ww along j_y (-w along j_z)
+  const C c73 = C(7.0 / 3.0);
+  out[1] = (a + px) * jx - c73 * smu[4] + (smu[11] * jy + smu[13] * jz) * ir0;
+  out[2] = (a + pyz + w) * jy - c73 * smu[6] + (smu[11] * jx + smu[12] * jz) * ir0;
+  out[3] = (a + pyz - w) * jz - c73 * smu[8] + (smu[12] * jy + smu[13] * jx) * ir0;
+}
+
+// Collision transpose of one node in the compute type: t = M^T nu, gsum_k = dJ/ds_k, through
+// the factored transforms (fmoments, fmt), which take fewer operations than the pair form
+// (FP32: 0.349 -> 0.340 s for the backward pass at 128^3 x 2000).
+template <class L, class C>
+LBM_HD void adjoint_plain(const C (&g)[L::Q], const C (&lp)[L::Q], const SweepArgs<C> &sa, C (&t)[L::Q],
+                          C (&gsum)[L::Q]) {
+  constexpr int Q = L::Q;
+  const C ir0 = sa.inv_rho0;
+  C m[Q], mu[Q];
+  fmoments<C>(L{}, g, m);
+  fmoments<C>(L{}, lp, mu);
+  const C jx = m[3], jy = m[5], jz = L::D == 3 ? m[7] : C(0);
+  C smu[Q], nu[Q];
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int k = 0; k < Q; ++k) {
+    if (Rows<L>::cons(k)) {
+      smu[k] = C(0);
+      mu[k] *= C(1.0 / row_norm2<L>(k));
+      continue;
+    }
+    smu[k] = sa.sn[k] * mu[k];                                      // s_k (M lambda')_k / |M_k|^2
+    mu[k] *= C(1.0 / row_norm2<L>(k));
+    gsum[k] = mu[k] * (meq(L{}, k, m[0], jx, jy, jz, ir0) - m[k]);   // d m'_k/d s_k
+    nu[k] = mu[k] - smu[k];                                         // (1 - s_k) mu_k
+  }
+  C dq[4];
+  meq_adjoint(L{}, smu, jx, jy, jz, ir0, dq);
+  nu[0] = mu[0] + dq[0];
+  nu[3] = mu[3] + dq[1];
+  nu[5] = mu[5] + dq[2];
+  if (L::D == 3) nu[7] = mu[7] + dq[3];
+  fmt<true, C>(L{}, nu, t);
+}
 
 // ---------------------------------------------------------------------------
 // The collision transpose of FP64 storage in block fixed point (fixed.cuh): the state's
@@ -15,8 +91,13 @@ namespace lbm {
 // products and the boundary terms are FP64.  Forward and backward pass over 40 steps:
 // D3Q19 96^3 33.1 -> 16.0 ms, 56^3 7.2 -> 3.5; D2Q9 96^2 x 100 2.45 -> 2.05.
 //
-// The adjoint populations are multiples of 2^(E_l - 53), E_l their largest exponent; sums
-// with M (up to 192 times the largest) fit 62 bits.  Scaled moments and results are
+// The adjoint populations are multiples of 2^(E_l - kAdjIn), E_l their largest exponent, as
+// fine as the largest row sum of M allows (16, 48 and 192 times the largest: 2^62, 2^61.6 and
+// 2^62.6, fx_mul's limit is 2^62.9).  dJ/ds takes the exact sums M lambda': on a smooth
+// adjoint field it consists of the small moments, and with entries in multiples of
+// 2^(E_l - 53) and moments of 2^(E_l - 57) its error was up to twice that of the FP64 form
+// (rms of a node's largest: D2Q9 4.6e-14, now 2.2e-15, FP64 4.8e-14; D3Q15 6.8e-14, 1.0e-14,
+// 3.6e-14; D3Q19 4.0e-14, 1.6e-14, 3.3e-14; tests/test_fixed_point_host.py).  Scaled moments and results are
 // multiples of 2^(E_l - 57), the largest adjoint value is below 2^58 of them, and 64 bits
 // hold 32 times that.  For every s in [0, 2] and |u_a| < 0.63 (deviations under rho0/16,
 // fx_block's range) results stay below 13 times the largest adjoint value and the factors of the
@@ -26,20 +107,31 @@ namespace lbm {
 // 38 and 22 for its factors, with a shift by 3, would reach 48.8).  tests/test_fixed_point_host.py
 // runs the extremes with overflow checks.  Nodes outside these ranges take the FP64 form.
 // ---------------------------------------------------------------------------
-constexpr int kAdjIn = 53, kAdjOut = 57;
+template <class L>
+constexpr int kAdjIn = L::Q == 9 ? 57 : (L::Q == 15 ? 55 : 54);
+constexpr int kAdjOut = 57;
 template <class L>
 constexpr int row_abs_sum(int k) {
   int s = 0;
   for (int i = 0; i < L::Q; ++i) s += L::M(k, i) < 0 ? -L::M(k, i) : L::M(k, i);
   return s;
 }
-// left shift of moment k before its products: its sum stays below 2^62
+// left shift of moment k before its products: its sum stays below 2^62 (2^62.6 for row e of D3Q19)
 template <class L>
 constexpr int adj_shift(int k) {
   int sh = 0;
-  while (row_abs_sum<L>(k) << (sh + 1) <= 256) ++sh;
+  while ((i64)row_abs_sum<L>(k) << (sh + 1) <= (i64)1 << (61 - kAdjIn<L>)) ++sh;
   return sh;
 }
+// what fx_mul takes: 2^62.9 = 1.866 x 2^62, with entries below 2^(kAdjIn + 1)
+template <class L>
+constexpr bool adj_sums_fit() {
+  for (int k = 0; k < L::Q; ++k)
+    if (100 * ((i64)row_abs_sum<L>(k) << adj_shift<L>(k)) > (i64)186 << (61 - kAdjIn<L>) || adj_shift<L>(k) > 7)
+      return false;
+  return true;
+}
+static_assert(adj_sums_fit<D2Q9>() && adj_sums_fit<D3Q15>() && adj_sums_fit<D3Q19>(), "moments of the adjoint fit fx_mul");
 // all rows' shifts, 3 bits each: a literal in device code
 template <class L>
 constexpr u64 adj_shifts() {
@@ -58,7 +150,7 @@ template <class L>
 inline FixedAdj fx_adj_args(const double *sn) {
   FixedAdj f{};
   for (int k = 0; k < L::Q; ++k) {
-    const int e = kAdjOut - kAdjIn - adj_shift<L>(k) + fx_fine<L>(k);
+    const int e = kAdjOut - kAdjIn<L> - adj_shift<L>(k) + fx_fine<L>(k);
     f.inv_n[k] = fx_coef(ldexp(1.0 / row_norm2<L>(k), e));
     f.s_n[k] = L::conserved(k) ? FixedCoef{0, 0} : fx_coef(ldexp(sn[k], e));
   }
@@ -126,10 +218,14 @@ LBM_HD void fx_adj_back(D3Q19, const i64 (&nu)[19], i64 (&t)[19]) {
   for (int i = 1; i < 19; ++i) t[i] += i < 7 ? face : edge;
 }
 
-// Collision transpose of one node: t = M^T nu from g and lambda' (lp), and gsum_k =
-// mu_k / |M_k|^2 (m^eq_k - m_k) over -fx_neq_scale 2^-fx_fine (products in FP64: m_k - m^eq_k is
-// often small, and a product in the moments' units would lose its digits); false if
-// the node is outside the integer ranges.
+// dJ/ds_k over the gsum_k of fx_adjoint
+template <class L>
+LBM_HD constexpr double fx_gsum_scale(int k) { return L::conserved(k) ? 0.0 : -fx_neq_scale<L>(k) / row_norm2<L>(k); }
+
+// Collision transpose of one node: t = M^T nu from g and lambda' (lp), and gsum_k = mu_k |M_k|^2
+// (m_k - m^eq_k) / fx_neq_scale, the exact sum M lambda' times the relaxed moment (products in
+// FP64: m_k - m^eq_k is often small, and a product in the moments' units would lose its
+// digits); false if the node is outside the integer ranges.
 template <class L>
 LBM_HD bool fx_adjoint(const double (&g)[L::Q], const double (&lp)[L::Q], const FixedArgs &fx,
                        const FixedAdj &fa, double (&t)[L::Q], double (&gsum)[L::Q]) {
@@ -158,7 +254,7 @@ LBM_HD bool fx_adjoint(const double (&g)[L::Q], const double (&lp)[L::Q], const 
 #ifdef __CUDA_ARCH__
 #pragma unroll
 #endif
-  for (int i = 0; i < L::Q; ++i) v[i] = fx_from<kAdjIn>(lp[i], El);
+  for (int i = 0; i < L::Q; ++i) v[i] = fx_from<kAdjIn<L>>(lp[i], El);
   i64 nu[L::Q], smu[L::Q];
   {
     i64 mu[L::Q];
@@ -172,7 +268,7 @@ LBM_HD bool fx_adjoint(const double (&g)[L::Q], const double (&lp)[L::Q], const 
       smu[k] = 0;
       if (!Rows<L>::cons(k)) {
         smu[k] = fx_mul(m, fa.s_n[k]);
-        gsum[k] = fx_to<kAdjOut>(nu[k], El) * fx_to<kFxTop<L>>(n[k], Eg);
+        gsum[k] = fx_to<kAdjIn<L>>(mu[k], El) * fx_to<kFxTop<L>>(n[k], Eg);
         nu[k] -= smu[k];
       }
     }

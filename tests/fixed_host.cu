@@ -1,12 +1,12 @@
 // fixed_host.cu -- runs the library's fixed-point arithmetic (fixed.cuh, fixed_adjoint.cuh)
 // on the host for tests/test_fixed_point_host.py.
 //
-//   fixed_host collide|adjoint D2Q9|D3Q15|D3Q19 < in > out
+//   fixed_host collide|adjoint|adjoint_fp64 D2Q9|D3Q15|D3Q19 < in > out
 //
 // in:  doubles n, rho0, F[3] (the force on the momentum rows), s[19], then per node g[Q]
-//      and, for adjoint, lambda'[Q].
+//      and, for the adjoint forms, lambda'[Q].
 // out: per node 1.0 where the fixed-point form covers it (else 0.0), then for collide g'[Q]
-//      in fixed point and g'[Q] in FP64, for adjoint the transpose t[Q] and dJ/ds[Q].
+//      in fixed point and g'[Q] in FP64, for the adjoint forms the transpose t[Q] and dJ/ds[Q].
 #include <stdio.h>
 #include <string.h>
 
@@ -20,7 +20,7 @@ static bool get(double *p, size_t n) { return fread(p, sizeof(double), n, stdin)
 static void put(const double *p, size_t n) { fwrite(p, sizeof(double), n, stdout); }
 
 template <class L>
-static int run(bool adjoint) {
+static int run(bool adjoint, bool fp64) {
   double head[5], s[19];
   if (!get(head, 5) || !get(s, 19)) return 2;
   SweepArgs<double> a{};
@@ -33,10 +33,12 @@ static int run(bool adjoint) {
     double g[L::Q], x[L::Q], y[L::Q] = {}, z[L::Q] = {};
     if (!get(g, L::Q) || (adjoint && !get(x, L::Q))) return 2;
     bool ok;
-    if (adjoint) {
+    if (adjoint && fp64) {
+      ok = true;
+      adjoint_plain<L, double>(g, x, a, y, z);
+    } else if (adjoint) {
       ok = fx_adjoint<L>(g, x, a.fx, fa, y, z);
-      for (int k = 0; k < L::Q; ++k)
-        z[k] = L::conserved(k) ? 0.0 : z[k] * -fx_neq_scale<L>(k) / (1 << fx_fine<L>(k));
+      for (int k = 0; k < L::Q; ++k) z[k] *= fx_gsum_scale<L>(k);
     } else {
       ok = collide_fixed<L>(g, y, a);
       collide_plain<L>(g, z, a);
@@ -51,8 +53,8 @@ static int run(bool adjoint) {
 
 int main(int argc, char **argv) {
   if (argc != 3) return 2;
-  const bool adjoint = strcmp(argv[1], "adjoint") == 0;
-  if (strcmp(argv[2], "D2Q9") == 0) return run<D2Q9>(adjoint);
-  if (strcmp(argv[2], "D3Q15") == 0) return run<D3Q15>(adjoint);
-  return run<D3Q19>(adjoint);
+  const bool fp64 = strcmp(argv[1], "adjoint_fp64") == 0, adjoint = fp64 || strcmp(argv[1], "adjoint") == 0;
+  if (strcmp(argv[2], "D2Q9") == 0) return run<D2Q9>(adjoint, fp64);
+  if (strcmp(argv[2], "D3Q15") == 0) return run<D3Q15>(adjoint, fp64);
+  return run<D3Q19>(adjoint, fp64);
 }

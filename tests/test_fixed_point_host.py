@@ -189,3 +189,32 @@ def test_collision_error_is_below_that_of_fp64(host, lattice, s_nu):
         rms = [float(np.sqrt((half_ulps(x - want, g) ** 2).mean())) for x in (fixed, plain)]
         print("%s s_nu %g state %s: rms %.2f fixed point, %.2f FP64 (half ulps)" % (lattice, s_nu, state, *rms))
         assert ok.all() and rms[0] <= rms[1]
+
+
+@pytest.mark.parametrize("lattice", ["D2Q9", "D3Q15", "D3Q19"])
+@pytest.mark.parametrize("s_nu", [0.5, 1.0, 1.9])
+@pytest.mark.parametrize("field", ["random", "smooth", "density"])
+def test_transpose_error_is_below_that_of_fp64(host, lattice, s_nu, field):
+    # smooth fields, whose moments other than rho and j are small, are what an adjoint
+    # settles to; dJ/ds is made of just those small moments
+    lat = OL.BY_NAME[lattice]
+    rng = np.random.default_rng(8)
+    s = W.relaxation_rates(lattice, s_nu)
+    for state in STATES:
+        g = near_equilibrium(lat, rng, *state)
+        n = g.shape[1]
+        lp = rng.standard_normal((lat.Q, n))
+        if field == "smooth":
+            lp = lat.e @ rng.standard_normal((3, n)) + 1e-3 * lp
+        elif field == "density":
+            lp = rng.standard_normal(n) + 0.1 * (lat.e @ rng.standard_normal((3, n))) + 1e-3 * lp
+        want, want_s = transpose(lat, s, 1.0, g, lp)
+        size = np.abs(want_s).max(0)
+        rms = []
+        for op in ("adjoint", "adjoint_fp64"):
+            ok, t, gs = host(op, lat, s, 1.0, np.zeros(3), g, lp)
+            assert ok.all()
+            rms += [float(np.sqrt((half_ulps(t - want, lp) ** 2).mean())), float(np.sqrt((((gs - want_s) / size) ** 2).mean()))]
+        print("%s s_nu %g %s, state %s: lambda %.2f fixed point, %.2f FP64 (half ulps); dJ/ds %.2e, %.2e"
+              % (lattice, s_nu, field, state, rms[0], rms[2], rms[1], rms[3]))
+        assert rms[0] <= rms[2] and rms[1] <= rms[3]
