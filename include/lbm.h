@@ -256,8 +256,7 @@ int lbm_set_link_values(lbm_ctx *ctx, const double *q, const double *uw);
  *             lbm_set_geometry, or NULL.
  *   grad_uw   3*n_links doubles: dJ/dphi per link, or NULL.
  * The adjoint computes in double for LBM_F64 and in float otherwise; gradients
- * are accumulated in double (a link's, from sums over at most sqrt(n_steps) steps in
- * the compute type).  Memory: about (n_steps/checkpoint_every +
+ * are accumulated in double.  Memory: about (n_steps/checkpoint_every +
  * checkpoint_every + 3) population arrays, n_steps + 3 where every state is kept,
  * held in the context after a successful call and reused (grown when needed) by later
  * calls; lbm_destroy releases it. */

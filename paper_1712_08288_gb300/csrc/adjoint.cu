@@ -137,12 +137,26 @@ __global__ void loss_kernel(AuxArgs a, bool odd, const uint8_t *mask, const doub
 //   dJ/dq   = b sum_t lambda_i (A' f_d + B' f'_i + C' f'_d) + b W' sum_t a(t) lambda_i,
 //   dJ/dphi = b 2 w_i rho0 e_i / ((1 + l) c_s^2) sum_t a(t) lambda_i,
 // with ' = d/dq.  The kernel accumulates only sum_t a(t) lambda_i and the first sum,
-// per link and in the compute type; the host folds in the other factors in FP64.
+// per link in FP64, with reductions that L2 carries out (one thread adds to a link in a
+// step, so their order is fixed); the host folds in the other factors.  FP32 sums would
+// lose digits with the length of the run or need a flush to FP64 every sqrt(T) steps, a
+// launch each (forward and backward pass, D3Q19 FP32 32^3 x 100: 1.66 ms with flushes, 1.57
+// so; 64^3 x 144 4.33 and 4.32; D2Q9 FP64 96^2 x 100 1.65 and 1.62); FP32 sums that carry
+// their rounding (two-sum) spill: 64^3 4.88.
 struct AdjGeo {
   const void *dcoef;          // LinkCoef<C> per link: (A', B', C', 0)
-  void *acc;                  // 2 C per link: sum lambda_i, sum lambda_i (A' g_d + B' g'_i + C' g'_d)
+  double *acc;                // 2 per link: sum lambda_i, sum lambda_i (A' g_d + B' g'_i + C' g'_d)
   FixedAdj fx;                // FP64 storage: constants of the fixed-point collision transpose
 };
+
+// v in FP64: by its bits for normal numbers (a conversion instruction issues for 64 cycles)
+__device__ __forceinline__ double to_f64(double v) { return v; }
+__device__ __forceinline__ double to_f64(float v) {
+  const unsigned b = __float_as_uint(v);
+  if (((b >> 23) & 0xffu) - 1u < 254u)
+    return __hiloint2double((int)((b & 0x80000000u) | (((b >> 3) & 0x0fffffffu) + 0x38000000u)), (int)(b << 29));
+  return v == 0.0f ? 0.0 : (double)v;
+}
 
 // position of row k among the non-conserved rows
 template <class L>
@@ -234,9 +248,9 @@ __global__ void __launch_bounds__(kAdjThreads, sizeof(C) == 4 ? LBM_ADJ_MINB_F32
           }
           // deviations suffice: A' + B' + C' = 0 removes the w_i rho0 parts
           const LinkCoef<C> dc = static_cast<const LinkCoef<C> *>(ag.dcoef)[k];
-          C *acc = static_cast<C *>(ag.acc) + 2 * (long long)k;
-          acc[0] += av * sa.wfac;           // W and its derivatives carry the step's factor
-          acc[1] += av * (dc.a * g[dd] + dc.bb * gp[i] + dc.c * gp[dd]);
+          double *acc = ag.acc + 2 * (long long)k;
+          atomic_add_double(acc, to_f64(av * sa.wfac));           // W and its derivatives carry the step's factor
+          atomic_add_double(acc + 1, to_f64(av * (dc.a * g[dd] + dc.bb * gp[i] + dc.c * gp[dd])));
         }
       }
     }
@@ -374,14 +388,13 @@ __global__ void __launch_bounds__(kAdjThreads, sizeof(C) == 4 ? 6 : 3)
   }
 }
 
-// add the per-link sums of the last steps to the FP64 totals and clear them
-template <class C>
-__global__ void link_flush_kernel(C *acc, double *tot, long long n) {
+// add the links' sums of the last steps to their totals and clear them
+__global__ void link_flush_kernel(double *acc, double *tot, long long n) {
   wait_for_previous();
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n;
        j += (long long)gridDim.x * blockDim.x) {
-    tot[j] += (double)acc[j];
-    acc[j] = C(0);
+    tot[j] += acc[j];
+    acc[j] = 0.0;
   }
 }
 
@@ -452,7 +465,7 @@ cudaError_t launch_loss(int lattice, int precision, const AuxArgs &a, bool odd, 
 
 cudaError_t launch_adjoint_step(int lattice, int precision, const SweepArgs<double> &a64,
                                 const SweepArgs<float> &a32, const AuxArgs &a, const void *dcoef,
-                                void *link_acc, const void *f, const void *lam_in, void *lam_out,
+                                double *link_acc, const void *f, const void *lam_in, void *lam_out,
                                 double *gs_part, cudaStream_t st) {
   AdjGeo ag{dcoef, link_acc, {}};
   const unsigned blocks = (unsigned)adjoint_partial_blocks(a.N);
@@ -488,13 +501,10 @@ cudaError_t launch_recompute_step(int lattice, int precision, const SweepArgs<do
   });
 }
 
-cudaError_t launch_link_flush(int precision, void *link_acc, double *tot, long long n,
-                              cudaStream_t st) {
+cudaError_t launch_link_flush(double *link_acc, double *tot, long long n, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int blocks = (int)std::min<long long>((n + 255) / 256, 152 * 8);
-  if (precision == 0)
-    return launch_early(link_flush_kernel<double>, blocks, 256, 0, st, static_cast<double *>(link_acc), tot, n);
-  return launch_early(link_flush_kernel<float>, blocks, 256, 0, st, static_cast<float *>(link_acc), tot, n);
+  return launch_early(link_flush_kernel, blocks, 256, 0, st, link_acc, tot, n);
 }
 
 long long adjoint_partial_blocks(long long N) { return (N + kAdjThreads - 1) / kAdjThreads; }

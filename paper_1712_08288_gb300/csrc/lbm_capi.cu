@@ -1088,7 +1088,7 @@ int adjoint_forward_impl(lbm_ctx *c, int n_steps, int checkpoint_every, const ui
   ADJ_CUDA(adj_ws_get(c, kUt, sizeof(double) * c->N * c->D, (void **)&dut));
   ADJ_CUDA(adj_ws_get(c, kGs, sizeof(double) * 19, &p));
   ADJ_CUDA(adj_ws_get(c, kTot, sizeof(double) * 2 * nl1, &p));
-  ADJ_CUDA(adj_ws_get(c, kAcc, csize * 2 * nl1, &p));
+  ADJ_CUDA(adj_ws_get(c, kAcc, sizeof(double) * 2 * nl1, &p));
   ADJ_CUDA(adj_ws_get(c, kDcoef, csize * 4 * nl1, &p));
   ADJ_CUDA(adj_ws_get(c, kJ, sizeof(double), (void **)&dJ));
   ADJ_CUDA(adj_ws_get(c, kGpart, sizeof(double) * c->Q * pblocks, &p));
@@ -1171,7 +1171,8 @@ int adjoint_backward_impl(lbm_ctx *c, double *grad_s, double *grad_q, double *gr
   char *fin = static_cast<char *>(c->adj_ws[kFin].first);
   char *lam0 = static_cast<char *>(c->adj_ws[kLam0].first), *lam1 = static_cast<char *>(c->adj_ws[kLam1].first);
   double *dgs = static_cast<double *>(c->adj_ws[kGs].first), *dtot = static_cast<double *>(c->adj_ws[kTot].first);
-  void *acc = c->adj_ws[kAcc].first, *dcoef = c->adj_ws[kDcoef].first;
+  double *acc = static_cast<double *>(c->adj_ws[kAcc].first);
+  void *dcoef = c->adj_ws[kDcoef].first;
   double *gpart = static_cast<double *>(c->adj_ws[kGpart].first);
   cudaStream_t st = c->stream;
   tp.valid = false;   // reset below once the state is restored
@@ -1186,7 +1187,7 @@ int adjoint_backward_impl(lbm_ctx *c, double *grad_s, double *grad_q, double *gr
   ADJ_CUDA(cudaMemsetAsync(gpart, 0, sizeof(double) * c->Q * pblocks, st));
   ADJ_CUDA(cudaMemsetAsync(dgs, 0, sizeof(double) * 19, st));
   ADJ_CUDA(cudaMemsetAsync(dtot, 0, sizeof(double) * 2 * nl1, st));
-  ADJ_CUDA(cudaMemsetAsync(acc, 0, csize * 2 * nl1, st));
+  ADJ_CUDA(cudaMemsetAsync(acc, 0, sizeof(double) * 2 * nl1, st));
   // d(A, B, C)/dq per link (Eq. 2.10 with l = c0 + c1 q + c2 q^2), device order
   std::vector<double> hdc(4 * nl1, 0.0);
   for (long long k = 0; k < nl; ++k) {
@@ -1224,9 +1225,9 @@ int adjoint_backward_impl(lbm_ctx *c, double *grad_s, double *grad_q, double *gr
   // when an earlier backward pass has overwritten the states the forward pass left),
   // then step back through it
   char *lin = lam0, *lout = lam1;
-  // The links' sums are held in the compute type and added to the FP64 totals after every
-  // segment and at least every sqrt(T) steps: with every state kept the run is one segment,
-  // and sequential FP32 sums over 20000 steps would keep 5 digits instead of 7.
+  // The links' sums run in FP64.  Those of FP64 storage go to totals after every segment and
+  // at least every sqrt(T) steps, which rounds less than one sum over the run.
+  const bool f64 = c->precision == LBM_F64;
   const long long flush_every = (long long)std::ceil(std::sqrt((double)T));
   long long unflushed = 0;
   const bool last_saved = tp.last_saved;
@@ -1257,8 +1258,8 @@ int adjoint_backward_impl(lbm_ctx *c, double *grad_s, double *grad_q, double *gr
       ADJ_CUDA(launch_adjoint_step(c->lattice, c->precision, c->a64, c->a32, aux_args(c), dcoef,
                                    acc, at(r), lin, lout, gpart, st));
       std::swap(lin, lout);
-      if (++unflushed == flush_every || r == 0) {
-        ADJ_CUDA(launch_link_flush(c->precision, acc, dtot, 2 * nl, st));
+      if (f64 ? ++unflushed == flush_every || r == 0 : sgm == 0 && r == 0) {
+        ADJ_CUDA(launch_link_flush(acc, dtot, 2 * nl, st));
         unflushed = 0;
       }
     }

@@ -219,11 +219,10 @@ cudaError_t launch_two_node(int lattice, int precision, const SweepArgs<double> 
                             const TwoNodeLink *tn, long long n_tn, void *delta, cudaStream_t st);
 
 // one step of the adjoint sweep: lambda(t) from lambda(t+1) and the pre-collision
-// state f (natural layout, compute type); per-link sums into link_acc (2 compute-type
-// values per link), dJ/ds into the per-block partial records
+// state f (natural layout, compute type); per-link sums into link_acc (2 per link), dJ/ds into the per-block partial records
 cudaError_t launch_adjoint_step(int lattice, int precision, const SweepArgs<double> &a64,
                                 const SweepArgs<float> &a32, const AuxArgs &a, const void *dcoef,
-                                void *link_acc, const void *f, const void *lam_in, void *lam_out,
+                                double *link_acc, const void *f, const void *lam_in, void *lam_out,
                                 double *gs_part, cudaStream_t st);
 // f(t+1) from f(t), both natural layout in the compute type (push form, same
 // arithmetic as the sweep); for recomputing adjoint segments of FP64 / FP32 storage
@@ -231,8 +230,7 @@ cudaError_t launch_recompute_step(int lattice, int precision, const SweepArgs<do
                                   const SweepArgs<float> &a32, const AuxArgs &a, const void *fin,
                                   void *fout, cudaStream_t st);
 // tot[j] += link_acc[j], link_acc[j] = 0 for j < n
-cudaError_t launch_link_flush(int precision, void *link_acc, double *tot, long long n,
-                              cudaStream_t st);
+cudaError_t launch_link_flush(double *link_acc, double *tot, long long n, cudaStream_t st);
 // per-block partial sums of dJ/ds (Q doubles per block), reduced by launch_adjoint_finish
 long long adjoint_partial_blocks(long long N);
 cudaError_t launch_adjoint_finish(int lattice, const double *gs_part, long long n_blocks,

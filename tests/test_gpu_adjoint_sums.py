@@ -2,13 +2,13 @@
 
 16-bit storage recomputes a segment with the sweep itself, so the states and the adjoint of a
 run are the same bit for bit for every checkpoint interval, and the gradients of two intervals
-differ only in how the FP32 sums over the steps are grouped before FP64 takes them.
+differ only in how the sums over the steps are rounded.
 
 An interval of one step adds every term in FP64.
 
 Tolerance: in a slowly decaying channel the terms of a link keep their sign and size, so n
 sequential FP32 additions are off by at most n roundings of 2^-25 of a sum that is on
-average half the result: n 2^-26, 3.7e-6 for the 245 steps that are added up in FP32
+average half the result: n 2^-26, 3.7e-6 where 245 steps, sqrt(T), are added up in FP32 before FP64 takes them
 (2e-7 where the roundings are random).  Over all 60000 steps the same bound is 9e-4.
 """
 
