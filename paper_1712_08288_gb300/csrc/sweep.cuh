@@ -267,10 +267,10 @@ template <class L, class C, class T = C>
 __device__ __forceinline__ bool collide(const C (&g)[L::Q], C (&gp)[L::Q], const SweepArgs<C> &a) {
   // The factored form where the sweep is bound by instruction issue: 16-bit storage (half
   // the bytes of FP32, the same instructions; 8 % faster) and the nodes that FP64
-  // storage does not cover in fixed point.  FP32 storage is bound by memory traffic, runs
-  // at the same speed with either form, and keeps the generic form, whose rounding
-  // tracks FP64 closer (E_r 0.2 % from FP64 after 20000 steps, against 2.3 % with
-  // the factored form).
+  // storage does not cover in fixed point.  FP32 storage, bound by the latency of its
+  // loads as much as by issue, runs at the same speed with either form, and keeps the
+  // generic form, whose rounding tracks FP64 closer (E_r 0.2 % from FP64 after 20000
+  // steps, against 2.3 % with the factored form).
   if constexpr (sizeof(C) == 8) {
     if (collide_fixed<L>(g, gp, a)) return false;
   }
