@@ -140,8 +140,8 @@ __global__ void loss_kernel(AuxArgs a, bool odd, const uint8_t *mask, const doub
 // per link in FP64, with reductions that L2 carries out (one thread adds to a link in a
 // step, so their order is fixed); the host folds in the other factors.  FP32 sums would
 // lose digits with the length of the run or need a flush to FP64 every sqrt(T) steps, a
-// launch each (forward and backward pass, D3Q19 FP32 32^3 x 100: 1.66 ms with flushes, 1.57
-// so; 64^3 x 144 4.33 and 4.32; D2Q9 FP64 96^2 x 100 1.65 and 1.62); FP32 sums that carry
+// launch each (forward and backward pass, D3Q19 FP32 32^3 x 100: 1.66 ms with flushes, 1.50
+// so; 64^3 x 144 4.33 and 4.17; D2Q9 FP64 96^2 x 100 1.65 and 1.61); FP32 sums that carry
 // their rounding (two-sum) spill: 64^3 4.88.
 struct AdjGeo {
   const void *dcoef;          // LinkCoef<C> per link: (A', B', C', 0)
@@ -149,14 +149,8 @@ struct AdjGeo {
   FixedAdj fx;                // FP64 storage: constants of the fixed-point collision transpose
 };
 
-// v in FP64: by its bits for normal numbers (a conversion instruction issues for 64 cycles)
 __device__ __forceinline__ double to_f64(double v) { return v; }
-__device__ __forceinline__ double to_f64(float v) {
-  const unsigned b = __float_as_uint(v);
-  if (((b >> 23) & 0xffu) - 1u < 254u)
-    return __hiloint2double((int)((b & 0x80000000u) | (((b >> 3) & 0x0fffffffu) + 0x38000000u)), (int)(b << 29));
-  return v == 0.0f ? 0.0 : (double)v;
-}
+__device__ __forceinline__ double to_f64(float v) { return fx_widen(v); }
 
 // position of row k among the non-conserved rows
 template <class L>

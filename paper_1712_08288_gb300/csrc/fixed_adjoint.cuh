@@ -8,6 +8,38 @@
 
 namespace lbm {
 
+LBM_HD unsigned fx_bits(float x) {
+#ifdef __CUDA_ARCH__
+  return __float_as_uint(x);
+#else
+  unsigned b;
+  memcpy(&b, &x, 4);
+  return b;
+#endif
+}
+LBM_HD double fx_double(unsigned hi, unsigned lo) {
+#ifdef __CUDA_ARCH__
+  return __hiloint2double((int)hi, (int)lo);
+#else
+  const u64 b = ((u64)hi << 32) | lo;
+  double x;
+  memcpy(&x, &b, 8);
+  return x;
+#endif
+}
+
+// v in FP64 by its bits, without the conversion instruction (64 issue cycles): the exponent
+// moves by 896, subnormal numbers are scaled by 2^64 first, infinities and NaN keep the
+// largest exponent.  Straight-line: a branch to the conversion for the rare values spills the
+// adjoint step's registers (D3Q19 FP32, 64^3 x 144 steps: 4.35 ms, 4.17 so, 4.23 converted).
+LBM_HD double fx_widen(float v) {
+  const bool tiny = fabsf(v) < 1.1754944e-38f;
+  const unsigned b = fx_bits(tiny ? v * 1.8446744073709552e19f : v);
+  const unsigned bias = (b & 0x7f800000u) == 0x7f800000u ? 0x70000000u : (tiny ? 0x34000000u : 0x38000000u);
+  const unsigned hi = (b & 0x7fffffffu) != 0u ? ((b >> 3) & 0x0fffffffu) + bias : 0u;
+  return fx_double(hi | (b & 0x80000000u), b << 29);
+}
+
 // sum_k smu_k * d meq_k / d(rho, j_x, j_y, j_z) for the equilibrium moments of
 // meq() (deviation form), smu_k = s_k mu_k on the non-conserved rows
 template <class C>

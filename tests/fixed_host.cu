@@ -3,6 +3,8 @@
 //
 //   fixed_host collide|adjoint|adjoint_fp64 D2Q9|D3Q15|D3Q19 < in > out
 //
+//   fixed_host widen any < floats > doubles (fx_widen of each)
+//
 // in:  doubles n, rho0, F[3] (the force on the momentum rows), s[19], then per node g[Q]
 //      and, for the adjoint forms, lambda'[Q].
 // out: per node 1.0 where the fixed-point form covers it (else 0.0), then for collide g'[Q]
@@ -53,6 +55,14 @@ static int run(bool adjoint, bool fp64) {
 
 int main(int argc, char **argv) {
   if (argc != 3) return 2;
+  if (strcmp(argv[1], "widen") == 0) {
+    float v;
+    while (fread(&v, sizeof v, 1, stdin) == 1) {
+      const double d = fx_widen(v);
+      put(&d, 1);
+    }
+    return 0;
+  }
   const bool fp64 = strcmp(argv[1], "adjoint_fp64") == 0, adjoint = fp64 || strcmp(argv[1], "adjoint") == 0;
   if (strcmp(argv[2], "D2Q9") == 0) return run<D2Q9>(adjoint, fp64);
   if (strcmp(argv[2], "D3Q15") == 0) return run<D3Q15>(adjoint, fp64);

@@ -54,6 +54,7 @@ def host(tmp_path_factory):
         out = np.frombuffer(r.stdout).reshape(n, 2 * lat.Q + 1)
         return out[:, 0] == 1.0, out[:, 1:1 + lat.Q].T, out[:, 1 + lat.Q:].T
 
+    run.exe = exe
     return run
 
 
@@ -218,3 +219,17 @@ def test_transpose_error_is_below_that_of_fp64(host, lattice, s_nu, field):
         print("%s s_nu %g %s, state %s: lambda %.2f fixed point, %.2f FP64 (half ulps); dJ/ds %.2e, %.2e"
               % (lattice, s_nu, field, state, rms[0], rms[2], rms[1], rms[3]))
         assert rms[0] <= rms[2] and rms[1] <= rms[3]
+
+
+def test_widening_by_bits_is_the_conversion(host):
+    rng = np.random.default_rng(3)
+    edges = [0, 1, 2, 0x7fffff, 0x800000, 0x800001, 0x3f800000, 0x7f7fffff, 0x7f800000, 0x7f800001, 0x7fc00000, 0x7fffffff]
+    bits = np.concatenate([np.array(edges, np.uint32), rng.integers(0, 1 << 31, 200000).astype(np.uint32),
+                           rng.integers(0, 1 << 23, 20000).astype(np.uint32)])
+    v = np.concatenate([bits, bits | np.uint32(1 << 31)]).view(np.float32)
+    r = subprocess.run([host.exe, "widen", "any"], input=v.tobytes(), stdout=subprocess.PIPE)
+    with np.errstate(invalid="ignore"):              # signalling NaN
+        got, want = np.frombuffer(r.stdout), v.astype(np.float64)
+    nan = np.isnan(want)
+    assert r.returncode == 0 and np.isnan(got[nan]).all()
+    assert np.array_equal(got[~nan].view(np.uint64), want[~nan].view(np.uint64))
