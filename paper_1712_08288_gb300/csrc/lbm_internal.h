@@ -121,7 +121,7 @@ struct FixedArgs {
   int max_exp;               // largest biased exponent of a block (below 0: none)
   int force_hi;              // high word of the largest force component
 };
-// the same for the adjoint's collision transpose (adjoint.cu)
+// the same for the adjoint's collision transpose (fixed_adjoint.cuh)
 struct FixedAdj {
   FixedCoef inv_n[19], s_n[19];
 };
